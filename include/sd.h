@@ -150,8 +150,9 @@ void sd_destroy(sd_handle *h);
 
 /* Positions r_i (n x 3 doubles), copied into the handle's FP64 state; also
  * refreshes the FP32 mirror the all-pairs kernel reads; with Verlet lists it also
- * builds the steps' near-pair list around the new positions, so a trajectory
- * resumed from positions read back continues bit for bit.  Non-finite values give
+ * builds the steps' near-pair list around the new positions (a small system's steps
+ * need none, see sd_step), so a trajectory resumed from positions read back continues
+ * bit for bit.  Non-finite values give
  * SD_ERR_NONFINITE (host pointers: from this call; device pointers: deferred). */
 sd_status sd_set_positions(sd_handle *h, const double *xyz, int on_device);
 sd_status sd_get_positions(sd_handle *h, double *xyz, int on_device);
@@ -167,7 +168,9 @@ sd_status sd_mobility_apply(sd_handle *h, const void *F, void *V, int dtype, int
 
 /* nsteps explicit Euler steps (Sec. 3.1): F = F(x_n), v = mu(x_n) F, x_{n+1} = x_n + dt v.
  * Position state is FP64.  Steps run as a replayed CUDA graph on the handle's stream
- * (asynchronous; errors surface at the next synchronising call).  nsteps >= 0. */
+ * (asynchronous; errors surface at the next synchronising call), or, for a small system
+ * with constant forces and dense_kernel AUTO (FP32C n <= 2048, FP64 n <= 1024), up to 512
+ * steps per cooperative kernel launch.  nsteps >= 0. */
 sd_status sd_step(sd_handle *h, double dt, int64_t nsteps);
 
 /* Row shards of the two calls above, for splitting one system over devices by

@@ -166,6 +166,23 @@ static cudaError_t launch_verlet_step(sd_handle *h, cudaStream_t st, double dt, 
     return e;
 }
 
+// Small systems run every product and step through one kernel (small.cu).  An injected
+// stall takes the kernels that copy in bulk.
+static bool use_small(const sd_handle *h) { return h->small.on && !h->inject_stall; }
+
+// The Verlet steps' list around the positions x64[cur].
+static sd_status build_list(sd_handle *h) {
+    SD_CUDA(cudaMemsetAsync(h->d_vl, 0, sizeof(int), h->stream));
+    SD_CUDA(cudaMemsetAsync(h->d_vl, 1, 1, h->stream));   // a rebuild request (bit 2 clear)
+    const double *x = h->x64[h->cur];
+    sd_status s = launch_check(launch_build_cells(h, h->stream, x, h->posm, h->xref), "neighbour list");
+    if (s == SD_OK)
+        s = launch_check(launch_near_collect(h, h->stream, x, h->posm.aos, h->F64, h->frcm.aos, true, true),
+                         "neighbour list");
+    h->list_set = s == SD_OK;
+    return s;
+}
+
 // x_out = x_in + dt mu(x_in) F(x_in); the cell-list build also writes the mirror of x_in.
 static cudaError_t launch_step(sd_handle *h, cudaStream_t st, double dt, const double *x_in, double *x_out) {
     if (h->verlet) return launch_verlet_step(h, st, dt, x_in, x_out);
@@ -245,6 +262,19 @@ static sd_status capture_steps(sd_handle *h, double dt, int cur, int k) {
 // profiler on, eager launches so that every kernel family gets its own event pair.
 static sd_status run_steps(sd_handle *h, double dt, int64_t nsteps) {
     int64_t left = nsteps;
+    if (use_small(h)) {
+        const int c = h->cur;
+        sd_status s = launch_check(launch_small(h, h->stream, OUT_EULER, h->x64[c], h->x64[1 - c], 0, h->F64, 0,
+                                                nullptr, dt, nsteps, 0, h->n),
+                                   "Euler steps");
+        if (s == SD_OK && (nsteps & 1)) h->cur = 1 - c;
+        h->cells_valid = false;
+        return s;
+    }
+    if (h->verlet && !h->list_set) {
+        sd_status s = build_list(h);
+        if (s != SD_OK) return s;
+    }
     auto replay = [&](int k) -> sd_status {
         const int c = h->cur;
         if (!h->gexec[k][c] || h->g_dt[k][c] != dt) {
@@ -285,6 +315,11 @@ static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int
     auto segx = [&](int64_t k) { return h->seg + static_cast<size_t>(k) * n3; };
     cudaError_t e = cudaSuccess;
     if (part == 0) {
+        if (use_small(h)) {
+            if (len > 1)
+                e = launch_small(h, st, OUT_EULER, segx(0), nullptr, n3, h->F64, 0, nullptr, dt, len - 1, 0, h->n);
+            return e;
+        }
         for (int64_t k = 0; k + 1 < len && e == cudaSuccess; ++k) e = launch_step(h, st, dt, segx(k), segx(k + 1));
         return e;
     }
@@ -517,12 +552,15 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
     if (h->n > 0) {
         e = dense_setup(h);
         if (e == cudaSuccess) e = vjp_setup(h);
+        if (e == cudaSuccess) e = small_setup(h);
         if (e != cudaSuccess) return fail(SD_ERR_CUDA, std::string("kernel set-up: ") + cudaGetErrorString(e));
         const int slots = std::max(h->geom.maxSlots, h->geomv.maxSlots);
         h->part_bytes = static_cast<size_t>(slots) * 3 * h->npad * sizeof(double);
         h->part2_bytes = static_cast<size_t>(h->geomv.maxSlots) * 3 * h->npad * sizeof(double);
         h->part = static_cast<double *>(dalloc(h, h->part_bytes));
         h->part2 = static_cast<double *>(dalloc(h, h->part2_bytes));
+        if (h->small.on && (!dalloc_t(h, h->small_sync, 3) || !dalloc_t(h, h->small_xch, 2 * n3)))
+            return fail(SD_ERR_OOM, "device allocation of the small systems' exchange");
         if (!h->part || !h->part2) return fail(SD_ERR_OOM, "device allocation of partial sums");
         if (h->geom.sym) {
             const size_t es = h->mode == MODE_FP64 ? sizeof(double) : sizeof(float);
@@ -538,6 +576,11 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_flag, 0, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_vl, 0, 3 * sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->d_vl, 0xff, sizeof(int), st);   // no list until positions are set
+    if (e == cudaSuccess && h->small_sync) {   // (the buffers' tags are 0; the first launch's are 1, 2, ...)
+        e = cudaMemsetAsync(h->small_sync, 0, 3 * sizeof(unsigned), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->small_sync, 1, 1, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->small_xch, 0, 2 * n3 * sizeof(ulonglong2), st);
+    }
     if (e == cudaSuccess && h->vn) e = cudaMemsetAsync(h->vn, 0, sizeof(*h->vn), st);
     for (int b = 0; b < 2 && e == cudaSuccess; ++b) e = cudaMemsetAsync(h->x64[b], 0, n3 * sizeof(double), st);
     for (Mirror *m : {&h->posm, &h->frcm, &h->frcam, &h->wam}) {
@@ -571,7 +614,7 @@ void sd_destroy(sd_handle *h) {
                     h->cl.cell, h->cl.key, h->cl.cnt, h->cl.start, h->cl.bsum, h->cl.sorted,
                     h->ckpt, h->seg, h->lam, h->gFacc, h->near64, h->d_flag, h->d_err,
                     h->near_ent, h->near_out, h->near_n, h->near_off, h->near_cnt, h->vlag, h->xref, h->d_vl,
-                    h->vent, h->voff, h->vcnt, h->vn};
+                    h->vent, h->voff, h->vcnt, h->vn, h->small_sync, h->small_xch};
     for (void *p : bufs) dfree(h, p);
     if (h->cap) cudaStreamDestroy(h->cap);
     if (h->side) cudaStreamDestroy(h->side);
@@ -620,14 +663,9 @@ sd_status sd_set_positions(sd_handle *h, const double *xyz, int on_device) {
         // and the steps' neighbour list is built afresh around them, so that a
         // trajectory resumed from positions read back continues bit for bit
         if (h->vlag) SD_CUDA(cudaMemsetAsync(h->vlag, 0, 3 * sizeof(double) * h->n, h->stream));
-        if (h->verlet) {
-            SD_CUDA(cudaMemsetAsync(h->d_vl, 0, sizeof(int), h->stream));
-            SD_CUDA(cudaMemsetAsync(h->d_vl, 1, 1, h->stream));   // a rebuild request (bit 2 clear)
-            s = launch_check(launch_build_cells(h, h->stream, h->x64[h->cur], h->posm, h->xref), "neighbour list");
-            if (s == SD_OK)
-                s = launch_check(launch_near_collect(h, h->stream, h->x64[h->cur], h->posm.aos, h->F64,
-                                                     h->frcm.aos, true, true),
-                                 "neighbour list");
+        h->list_set = false;
+        if (h->verlet && !use_small(h)) {   // (the small path needs no list)
+            s = build_list(h);
             if (s != SD_OK) return s;
         }
     }
@@ -723,6 +761,14 @@ static sd_status apply_rows(sd_handle *h, const void *F, void *V, int dtype, int
         Vd = out;
     }
     const TileWin w = row_window(h, row0, row1);
+    if (use_small(h)) {
+        sd_status s = launch_check(launch_small(h, h->stream, dtype == SD_DTYPE_F32 ? OUT_F32 : OUT_F64, h->x64[h->cur],
+                                                nullptr, 0, Fd, dtype == SD_DTYPE_F32, Vd, 0.0, 1, row0, row1),
+                                   "mobility product");
+        if (s != SD_OK || on_device) return s;
+        SD_CUDA(cudaMemcpyAsync(V, Vd, bytes_out, cudaMemcpyDeviceToHost, h->stream));
+        return sync_check(h);
+    }
     sd_status s = launch_check(launch_stage_forces(h, h->stream, Fd, dtype, 0, h->Fa64, h->frcam), "stage F");
     if (s == SD_OK) s = ensure_cells(h);
     if (s == SD_OK)
@@ -766,6 +812,15 @@ sd_status sd_step_rows(sd_handle *h, double dt, int32_t row0, int32_t row1) {
     cudaStream_t st = h->stream;
     const double *x_in = h->x64[h->cur];
     double *x_out = h->x64[1 - h->cur];
+    if (use_small(h)) {
+        sd_status s = launch_check(launch_small(h, st, OUT_EULER, h->x64[h->cur], x_out, 0, h->F64, 0, nullptr, dt, 1,
+                                                row0, row1),
+                                   "sharded step");
+        if (s != SD_OK) return s;
+        h->cur = 1 - h->cur;
+        h->cells_valid = false;
+        return SD_OK;
+    }
     const TileWin w = row_window(h, row0, row1);
     cudaError_t e = launch_build_cells(h, st, x_in, h->posm);
     if (e == cudaSuccess && !h->forces_const) e = launch_forces_rep(h, st, x_in);

@@ -1018,16 +1018,7 @@ static void launch_dense_t(sd_handle *h, cudaStream_t st, Mirror posm, Mirror fr
                                                                          dense_wd(h), w);
         return;
     }
-    PairConst2 c2{};
-    c2.c1 = pk2_host(h->pc.c1_f);
-    c2.c3 = pk2_host(h->pc.c3_f);
-    c2.m3c3 = pk2_host(h->pc.m3c3_f);
-    c2.r2min = h->pc.r2min_f;
-    for (int d = 0; d < 3; ++d) {
-        c2.negL[d] = pk2_host(-h->pc.Lf[d]);
-        c2.invL[d] = pk2_host(h->pc.invLf[d]);
-    }
-    c2.n = h->n;
+    const PairConst2 c2 = pair_const2(h->pc, h->n);
     const bool comp = h->mode == MODE_FP32C;
     if (g.sym) {
 #define SD_DS(TT, CC, BB, NN)                                                                                  \

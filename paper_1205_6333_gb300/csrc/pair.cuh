@@ -140,6 +140,20 @@ struct PairConst2 {
     int n;                 // particles (periodic kernels: tiles reaching index n clamp)
 };
 
+inline PairConst2 pair_const2(const PairConst &pc, int n) {
+    PairConst2 c{};
+    c.c1 = pk2_host(pc.c1_f);
+    c.c3 = pk2_host(pc.c3_f);
+    c.m3c3 = pk2_host(pc.m3c3_f);
+    c.r2min = pc.r2min_f;
+    for (int d = 0; d < 3; ++d) {
+        c.negL[d] = pk2_host(-pc.Lf[d]);
+        c.invL[d] = pk2_host(pc.invLf[d]);
+    }
+    c.n = n;
+    return c;
+}
+
 __device__ __forceinline__ f2 min_image2(f2 d, f2 negL, f2 invL) {
     const f2 magic = 0x4B4000004B400000ull;   // (1.5 2^23, 1.5 2^23)
     const f2 n = sub2(add2(mul2(d, invL), magic), magic);

@@ -132,6 +132,18 @@ struct Box {
     int periodic = 0;
 };
 
+// The one-launch path of small systems (small.cu): the launch shape.
+struct SmallGeom {
+    bool on = false;
+    int solo = 0;              // one CTA takes the system
+    int R = 1, nib = 0;        // targets per thread (FP32C), target blocks
+    int split = 1, jlen = 0;   // j-splits (CTAs per cluster), sources per split
+    int rows = 0;              // rows of a block that one CTA updates
+    int nbl = 1, wb = 1, iw = 32;   // target blocks per CTA, warps per block; FP64: targets per warp
+    int grid = 0;
+    size_t smem = 0;
+};
+
 // Hashed cell list over FP64 positions: cells of side h in unbounded dimensions
 // (no bounding box needed), nc[d] >= 3 cells of side L[d] / nc[d] >= h in a
 // periodic one (coordinates wrapped into [0, L)); H buckets (power of two),
@@ -226,6 +238,9 @@ struct sd_handle {
     void *jpart = nullptr;  size_t jpart_bytes = 0;   // symmetric kernels: source-side sums [tile][3][block],
                                                        // float (FP32 modes) or double (FP64)
     sd::DenseGeom geom{}, geomv{};
+    sd::SmallGeom small{};
+    unsigned *small_sync = nullptr;  // [3] words and
+    ulonglong2 *small_xch = nullptr; // [2][3 n] the position exchange of the small path (small.cu)
     int dense_occ = 0, vjp_occ = 0;
     int sym_nt = 128;   // threads per CTA of the symmetric kernel's chosen block shape
 
@@ -264,6 +279,7 @@ struct sd_handle {
     // the pairs within r_near + skin of the positions xref it was built from
     bool verlet = false;
     double skin = 0.0;
+    bool list_set = false;         // the list was built for some positions (the small path needs none)
     double list_cut = 0.0;         // cutoff of the Verlet list: max(r_near, r_c with repulsion, 3a with lubrication)
     double *xref = nullptr;        // [n*3] positions of the last build
     int *d_vl = nullptr;           // [0] rebuild request (bit 2: no list yet), [1] [2] check kernel's
@@ -334,6 +350,10 @@ cudaError_t launch_near_pairs(sd_handle *h, cudaStream_t st, const double *x64, 
 cudaError_t launch_epilogue(sd_handle *h, cudaStream_t st, int out, const double *x64, const void *posm,
                             const double *F64, const void *frcm, void *vout, double dt, double *x64n, int row0 = 0,
                             int row1 = -1, const EpiShard *shard = nullptr, bool vlist = false);
+// small.cu
+cudaError_t small_setup(sd_handle *h);
+cudaError_t launch_small(sd_handle *h, cudaStream_t st, int out, double *x0, double *x1, size_t stride, const void *F,
+                         int f32, void *vout, double dt, int64_t nsteps, int row0, int row1);
 // vjp.cu
 cudaError_t vjp_setup(sd_handle *h);
 cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm, double *partM,
