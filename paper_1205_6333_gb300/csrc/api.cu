@@ -466,6 +466,9 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
     pc.c1_d = 0.75 * a;
     pc.c3_d = 0.5 * a * a * a;
     pc.m3c3_d = -1.5 * a * a * a;
+    pc.k_d = pc.c3_d / pc.c1_d;
+    pc.m3k_d = -3.0 * pc.c3_d / pc.c1_d;
+    pc.invc1_d = 1.0 / pc.c1_d;
     pc.r2min_f = static_cast<float>(pc.r2min_d);
     pc.c1_f = static_cast<float>(pc.c1_d);
     pc.c3_f = static_cast<float>(pc.c3_d);

@@ -4,27 +4,17 @@
 //   v_i = mu0 [F_i + sum_{j != i in c} T^(r_i - r_j) F_j],  x_i <- x_i + dt v_i
 // (Sec. 2.2, Eq. rotneMobility; Sec. 3.1, steps 1 and 3).
 //
-// Work distribution: a persistent grid; every warp pops cluster tickets from a
-// global atomic counter (reset by a memset node before each step) and takes the
-// clusters in largest-first order (a longest-processing-time schedule), so the
-// small clusters fill the tail.  A warp stages its cluster in shared memory --
-// FP64 positions minus the cluster's first particle, rounded to FP32, so FP32
-// separations keep full relative precision and no FP64 near-pair pass is needed
-// -- and lane l owns particles l, l+32, ..., l+32(R-1), R = ceil(n/32).
-//
-// The j loop runs over 32-particle chunks in a lane-rotated order
-// (j = 32 jb + ((l + m) mod 32)), so a particle meets itself exactly at m = 0 of
-// its own chunk and that pair is skipped without a per-pair test.  Pairs use the
-// dense kernel's clamped pair term; a running minimum of r^2 flags overlaps
-// (r < 2a), and only then does a second pass replace the clamped terms of the
-// overlapping pairs by their exact values.  FP32C keeps per-lane (hi, lo)
-// accumulators in shared memory and folds each chunk's FP32 partial into them
-// with TwoSum.
+// Work distribution: a persistent grid pops tickets from a global atomic counter (reset by
+// a memset node before each step) and takes the clusters in largest-first order (a
+// longest-processing-time schedule), so the small clusters fill the tail.  Positions are
+// staged in shared memory relative to the cluster's first particle (FP64 differences, in
+// FP32C rounded to FP32, so FP32 separations keep full relative precision and no FP64
+// near-pair pass is needed).  FP32C has two kernels (one target's directed pairs per
+// thread; each unordered pair once), between which the autotuner picks; FP64 has one.
 #include <algorithm>
 #include <cmath>
 #include <new>
 #include <string>
-#include <type_traits>
 #include <tuple>
 #include <vector>
 
@@ -77,17 +67,6 @@ struct sd_batch {
 
 namespace sd {
 
-template <int MODE>
-struct BT {
-    using V4 = float4;
-    using S = float;
-};
-template <>
-struct BT<MODE_FP64> {
-    using V4 = dbl4;
-    using S = double;
-};
-
 struct BatchArgs {
     const int32_t *off, *order;
     const int32_t *qperm, *qcl, *cbeg, *cend, *canchor;
@@ -138,189 +117,142 @@ __device__ __forceinline__ void exact_pair(S dx, S dy, S dz, S fx, S fy, S fz, c
     oz = A * fz + s * dz;
 }
 
-template <int TENSOR, int MODE, int R>
-__device__ __forceinline__ void cluster_compute(const BatchArgs &a, int o, int n, double3 anchor,
-                                                const typename BT<MODE>::V4 *s_pos,
-                                                const typename BT<MODE>::V4 *s_frc, float *s_acc, int lane) {
-    using V4 = typename BT<MODE>::V4;
-    using S = typename BT<MODE>::S;
-    constexpr int TD = (TENSOR == T_OSEEN) ? T_OSEEN : T_RP;
-    constexpr bool COMP = (MODE == MODE_FP32C);
-    S xi[R], yi[R], zi[R], ax[R], ay[R], az[R];
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-        // slots beyond n sit far from everything (their results are discarded)
-        const V4 p = s_pos[lane + 32 * k];
-        const bool real = lane + 32 * k < n;
-        xi[k] = real ? S(p.x) : S(-1.0e15);
-        yi[k] = real ? S(p.y) : S(0);
-        zi[k] = real ? S(p.z) : S(0);
-        ax[k] = ay[k] = az[k] = S(0);
-        if (COMP)
-            for (int d = 0; d < 6; ++d) s_acc[(k * 6 + d) * 32 + lane] = 0.0f;
+// FP64 path: one CTA per cluster, each unordered pair once (mu_ij = mu_ji, Sec. 2.2).
+// Bound by the FP64 pipe (two operations a clock and SM), so the aim is fewer FP64
+// operations per pair: 35 per unordered pair here (profile64 and two directions of ten)
+// against 2 x 38 and an r^2 of its own per ordered pair in a kernel of one warp per cluster
+// with directed pairs (1,000 clusters of 4 .. 256: 3.1 ms a step; this one 0.79).
+//   * The cluster's positions (relative to its first particle) and forces are staged as six
+//     FP64 arrays, padded to whole blocks of 32 with far-away, force-free slots.  The warps
+//     take the block pairs (p, q), p <= q, in turn; every warp adds what a tile gives both
+//     its blocks to sums of its own, and the warps' sums are added in ascending order.
+//   * A tile (p, q), p < q: lane l holds target l of block q and meets source (l + m) mod 32
+//     of block p at step m; the source's running sum moves one lane down per step.  The
+//     last block is often partly filled: with w >= its particles a power of two, 32 / w
+//     groups of w lanes hold its targets, each group meets w of the 32 sources, and the tile
+//     takes w steps; the groups' target sums meet in a fixed shuffle tree.
+//   * A diagonal tile (width w) takes the steps m = 1 .. w / 2 (lanes l < w / 2 at the last).
+//   * Pairs closer than 2a leave the common path for the exact form, so nothing is clamped.
+template <int TENSOR>
+__device__ __forceinline__ void pair64_sym(const double (&t)[6], const double *__restrict__ s, bool on, const PairConst &c,
+                                           double (&A)[3], double (&J)[3], bool &coincident) {
+    const double dx = __dsub_rn(t[0], s[0]), dy = __dsub_rn(t[1], s[kMaxCluster]),
+                 dz = __dsub_rn(t[2], s[2 * kMaxCluster]);
+    const double fx = s[3 * kMaxCluster], fy = s[4 * kMaxCluster], fz = s[5 * kMaxCluster];
+    const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+    double a, b;
+    if (less_pos64(r2, c.r2min_d)) {   // rare (and idle lanes, which meet themselves)
+        a = b = 0.0;
+        if (on && r2 == 0.0 && TENSOR != T_RPY) {
+            coincident = true;
+        } else if (on) {
+            double da, db;
+            profile_exact<TENSOR>(r2, c, a, b, da, db);
+            a *= c.invc1_d;
+            b *= c.invc1_d;
+        }
+    } else {
+        profile64<TENSOR>(r2, c, a, b);
+        if (!on) a = b = 0.0;
     }
-    S mn = S(1e30);
-    const int nchunk = (n + 31) >> 5;
-    for (int jb = 0; jb < nchunk; ++jb) {
-        // m = 0: the diagonal slot k == jb meets itself; skip that pair only
-        {
-            const int j = 32 * jb + lane;
-            const V4 p = s_pos[j], f = s_frc[j];
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                if (k == jb) continue;
-                const S dx = xi[k] - p.x, dy = yi[k] - p.y, dz = zi[k] - p.z;
-                mn = fmin(mn, dx * dx + dy * dy + dz * dz);
-                if constexpr (MODE == MODE_FP64)
-                    pair_f64<TD>(xi[k], yi[k], zi[k], p, f, a.pc, ax[k], ay[k], az[k]);
-                else
-                    pair_f32<TD>(xi[k], yi[k], zi[k], p, f, a.pc, ax[k], ay[k], az[k]);
-            }
-        }
-        for (int m = 1; m < 32; ++m) {
-            const int j = 32 * jb + ((lane + m) & 31);
-            const V4 p = s_pos[j], f = s_frc[j];
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                if constexpr (MODE == MODE_FP64) {
-                    const double dx = xi[k] - p.x, dy = yi[k] - p.y, dz = zi[k] - p.z;
-                    mn = fmin(mn, dx * dx + dy * dy + dz * dz);
-                    pair_f64<TD>(xi[k], yi[k], zi[k], p, f, a.pc, ax[k], ay[k], az[k]);
-                } else {
-                    // the clamp in pair_f32 sees the same r^2; track it for the overlap test
-                    const float dx = __fsub_rn(xi[k], p.x), dy = __fsub_rn(yi[k], p.y), dz = __fsub_rn(zi[k], p.z);
-                    mn = fminf(mn, __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))));
-                    pair_f32<TD>(xi[k], yi[k], zi[k], p, f, a.pc, ax[k], ay[k], az[k]);
-                }
-            }
-        }
-        if constexpr (COMP) {
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                float *q = s_acc + k * 6 * 32 + lane;
-                float hx = q[0], hy = q[32], hz = q[64], lx = q[96], ly = q[128], lz = q[160];
-                fold2(hx, lx, ax[k]);
-                fold2(hy, ly, ay[k]);
-                fold2(hz, lz, az[k]);
-                q[0] = hx; q[32] = hy; q[64] = hz; q[96] = lx; q[128] = ly; q[160] = lz;
-                ax[k] = ay[k] = az[k] = 0.0f;
-            }
-        }
-    }
-    // per slot: compensated dense sum, exact terms for overlapping pairs (only
-    // when some lane saw r < 2a), self term mu_ii = mu0 I, Euler update in FP64
-    const bool overlap = __any_sync(0xffffffffu, mn < S(a.pc.r2min_d));
-    bool coincident = false;
-    const double m0 = a.pc.mu0, dt = a.dt;
-#pragma unroll
-    for (int k = 0; k < R; ++k) {
-        const int i = lane + 32 * k;
-        if (i >= n) continue;
-        double V0, V1, V2;
-        if constexpr (COMP) {
-            const float *q = s_acc + k * 6 * 32 + lane;
-            V0 = static_cast<double>(q[0]) + q[96];
-            V1 = static_cast<double>(q[32]) + q[128];
-            V2 = static_cast<double>(q[64]) + q[160];
-        } else {
-            V0 = ax[k];
-            V1 = ay[k];
-            V2 = az[k];
-        }
-        if (overlap) {
-            for (int j = 0; j < n; ++j) {
-                if (j == i) continue;
-                const V4 p = s_pos[j], f = s_frc[j];
-                S dx, dy, dz;
-                if constexpr (MODE == MODE_FP64) {
-                    dx = xi[k] - p.x; dy = yi[k] - p.y; dz = zi[k] - p.z;
-                } else {
-                    dx = __fsub_rn(xi[k], p.x); dy = __fsub_rn(yi[k], p.y); dz = __fsub_rn(zi[k], p.z);
-                }
-                const S r2 = dx * dx + dy * dy + dz * dz;
-                if (!(r2 < S(a.pc.r2min_d))) continue;
-                S cx = S(0), cy = S(0), cz = S(0);
-                if constexpr (MODE == MODE_FP64)
-                    pair_f64<TD>(xi[k], yi[k], zi[k], p, f, a.pc, cx, cy, cz);
-                else
-                    pair_f32<TD>(xi[k], yi[k], zi[k], p, f, a.pc, cx, cy, cz);
-                S ex, ey, ez;
-                exact_pair<TENSOR, S>(dx, dy, dz, S(f.x), S(f.y), S(f.z), a.pc, ex, ey, ez, coincident);
-                V0 += static_cast<double>(ex) - static_cast<double>(cx);
-                V1 += static_cast<double>(ey) - static_cast<double>(cy);
-                V2 += static_cast<double>(ez) - static_cast<double>(cz);
-            }
-        }
-        const size_t g = static_cast<size_t>(o + i);
-        const double vx = m0 * (V0 + a.F64[3 * g]);
-        const double vy = m0 * (V1 + a.F64[3 * g + 1]);
-        const double vz = m0 * (V2 + a.F64[3 * g + 2]);
-        const double nx = a.x64[3 * g] + dt * vx, ny = a.x64[3 * g + 1] + dt * vy, nz = a.x64[3 * g + 2] + dt * vz;
-        if (!isfinite(nx) || !isfinite(ny) || !isfinite(nz)) atomicOr(a.err, DEV_ERR_NONFINITE);
-        a.x64n[3 * g] = nx;
-        a.x64n[3 * g + 1] = ny;
-        a.x64n[3 * g + 2] = nz;
-    }
-    if (coincident) atomicOr(a.err, DEV_ERR_COINCIDENT);
-    (void)anchor;
+    const double u = __dmul_rn(b, __fma_rn(dz, fz, __fma_rn(dy, fy, __dmul_rn(dx, fx))));
+    A[0] = __fma_rn(u, dx, __fma_rn(a, fx, A[0]));
+    A[1] = __fma_rn(u, dy, __fma_rn(a, fy, A[1]));
+    A[2] = __fma_rn(u, dz, __fma_rn(a, fz, A[2]));
+    const double v = __dmul_rn(b, __fma_rn(dz, t[5], __fma_rn(dy, t[4], __dmul_rn(dx, t[3]))));
+    J[0] = __fma_rn(v, dx, __fma_rn(a, t[3], J[0]));
+    J[1] = __fma_rn(v, dy, __fma_rn(a, t[4], J[1]));
+    J[2] = __fma_rn(v, dz, __fma_rn(a, t[5], J[2]));
 }
 
-// FP64 path: one warp per cluster, scalar FP64 pairs.
-constexpr size_t kWarpStage = 2 * kMaxCluster * sizeof(dbl4);
+constexpr size_t batch64_smem(int warps) { return (6 + 3 * static_cast<size_t>(warps)) * kMaxCluster * sizeof(double); }
 
-template <int TENSOR>
-__global__ void batched_kernel(BatchArgs a) {
-    using V4 = dbl4;
-    extern __shared__ __align__(128) unsigned char smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned char *mine = smem + static_cast<size_t>(wid) * kWarpStage;
-    const V4 *frcm = static_cast<const V4 *>(a.frcm);
+template <int TENSOR, int NW>
+__global__ void __launch_bounds__(32 * NW) batched64_kernel(BatchArgs a) {
+    extern __shared__ __align__(16) double s_b64[];
+    __shared__ int s_t;
+    double *S = s_b64;                                     // [6][kMaxCluster]
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double *SUM = S + 6 * kMaxCluster;                     // [NW][3][kMaxCluster]
+    double *mine = SUM + static_cast<size_t>(wid) * 3 * kMaxCluster;
+    const dbl4 *frcm = static_cast<const dbl4 *>(a.frcm);
     for (;;) {
-        unsigned long long t = 0;
-        if (lane == 0) t = atomicAdd(a.ctr, 1ULL);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= static_cast<unsigned long long>(a.C)) break;
+        if (tid == 0) s_t = static_cast<int>(atomicAdd(a.ctr, 1ULL));
+        __syncthreads();
+        const int t = s_t;
+        if (t >= a.C) break;   // uniform over the CTA
         const int c = a.order[t];
-        const int o = a.off[c];
-        const int n = a.off[c + 1] - o;
-        if (n <= 0) continue;
-        if (n > kMaxCluster) {   // rejected at creation; never reached
-            if (lane == 0) atomicOr(a.err, DEV_ERR_QUEUE);
-            continue;
-        }
-        const double3 anchor = make_double3(a.x64[3 * o], a.x64[3 * o + 1], a.x64[3 * o + 2]);
-        const int R = (n + 31) >> 5;
-        V4 *s_pos = reinterpret_cast<V4 *>(mine);
-        V4 *s_frc = s_pos + kMaxCluster;
-        for (int p = lane; p < 32 * R; p += 32) {
-            V4 q, f;
+        const int o = a.off[c], n = min(a.off[c + 1] - o, kMaxCluster);   // (larger ones are rejected at creation)
+        const int nb = (n + 31) >> 5;
+        for (int p = tid; p < 32 * nb; p += 32 * NW) {
+            double v[6] = {1.0e15 * (p + 1), 0.0, 0.0, 0.0, 0.0, 0.0};
             if (p < n) {
                 const size_t g = static_cast<size_t>(o + p);
-                q.x = a.x64[3 * g] - anchor.x;
-                q.y = a.x64[3 * g + 1] - anchor.y;
-                q.z = a.x64[3 * g + 2] - anchor.z;
-                f = frcm[g];
-            } else {
-                // padding: far away (and far from the unused i-slots at -1e15), zero force
-                q.x = 1.0e15;
-                q.y = 0;
-                q.z = 0;
-                f.x = f.y = f.z = 0;
+                for (int d = 0; d < 3; ++d) v[d] = a.x64[3 * g + d] - a.x64[3 * static_cast<size_t>(o) + d];
+                const dbl4 f = frcm[g];
+                v[3] = f.x;
+                v[4] = f.y;
+                v[5] = f.z;
             }
-            q.w = 0;
-            f.w = 0;
-            s_pos[p] = q;
-            s_frc[p] = f;
+            for (int d = 0; d < 6; ++d) S[d * kMaxCluster + p] = v[d];
         }
-        __syncwarp();
-        switch (R) {
-#define SD_BR(RR) \
-    case RR: cluster_compute<TENSOR, MODE_FP64, RR>(a, o, n, anchor, s_pos, s_frc, nullptr, lane); break
-            SD_BR(1); SD_BR(2); SD_BR(3); SD_BR(4); SD_BR(5); SD_BR(6); SD_BR(7); SD_BR(8);
-#undef SD_BR
-            default: break;
+        for (int p = lane; p < 32 * nb; p += 32)
+            for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + p] = 0.0;
+        __syncthreads();
+        int wl = 32;   // width of the last block
+        while (wl > 2 && wl / 2 >= n - 32 * (nb - 1)) wl /= 2;
+        bool coincident = false;
+        const int noff = nb * (nb - 1) / 2;
+        // the off-diagonal tiles column by column from the first (full) ones, then the diagonal
+        for (int u = wid; u < noff + nb; u += NW) {
+            int p, q;
+            if (u < noff) {
+                q = 1;
+                while (q * (q + 1) / 2 <= u) ++q;
+                p = u - q * (q - 1) / 2;
+            } else {
+                p = q = u - noff;
+            }
+            const bool diag = p == q;
+            const int w = q == nb - 1 ? wl : 32, in = lane & (w - 1);
+            const int i = 32 * q + in;                                 // this lane's target
+            const int nxt = (lane & ~(w - 1)) | ((lane + 1) & (w - 1));
+            const double *src = S + 32 * p + (diag ? 0 : lane & ~(w - 1));
+            double T[6], A[3] = {0.0, 0.0, 0.0}, J[3] = {0.0, 0.0, 0.0};
+            for (int d = 0; d < 6; ++d) T[d] = S[d * kMaxCluster + i];
+            const int m0 = diag ? 1 : 0, m1 = diag ? w / 2 : w - 1;
+#pragma unroll 1
+            for (int m = m0; m <= m1; ++m) {
+                const bool on = !diag || (lane < w && (m < w / 2 || in < w / 2));
+                pair64_sym<TENSOR>(T, src + ((in + m) & (w - 1)), on, a.pc, A, J, coincident);
+                if (m < m1 || !diag)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) J[d] = __shfl_sync(0xffffffffu, J[d], nxt);
+            }
+            // off-diagonal: lane l holds source l of block p again; diagonal: source l + w / 2
+            const int sj = diag ? 32 * p + ((in + m1) & (w - 1)) : 32 * p + lane;
+            if (!diag || lane < w)
+                for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + sj] += J[d];
+            __syncwarp();
+            if (!diag)
+                for (int k = w; k < 32; k <<= 1)
+                    for (int d = 0; d < 3; ++d) A[d] += __shfl_xor_sync(0xffffffffu, A[d], k);
+            if (lane < w)
+                for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + i] += A[d];
+            __syncwarp();
         }
-        __syncwarp();
+        if (coincident) atomicOr(a.err, DEV_ERR_COINCIDENT);
+        __syncthreads();
+        for (int p = tid; p < 3 * n; p += 32 * NW) {
+            const int i = p / 3, d = p - 3 * i;
+            double V = SUM[d * kMaxCluster + i];
+            for (int k = 1; k < NW; ++k) V += SUM[(3 * k + d) * kMaxCluster + i];
+            const size_t g = 3 * static_cast<size_t>(o) + p;
+            const double nx = a.x64[g] + a.dt * (a.pc.mu0 * __fma_rn(a.pc.c1_d, V, S[(3 + d) * kMaxCluster + i]));
+            if (!isfinite(nx)) atomicOr(a.err, DEV_ERR_NONFINITE);
+            a.x64n[g] = nx;
+        }
+        __syncthreads();   // the stage and s_t are free for the next cluster
     }
 }
 
@@ -997,10 +929,10 @@ __global__ void __launch_bounds__(128, 3) batched_sym_kernel(BatchArgs a) {
     }
 }
 
-// Launch shapes: FP64 -- warps per CTA (one cluster per warp) x resident CTAs;
+// Launch shapes: FP64 -- warps per CTA (one cluster per CTA) x resident CTAs;
 // FP32C -- block of BT = 32 warps threads (R targets each) x resident CTAs.
 static size_t shape_smem(int mode, const BatchShape &sh) {
-    if (mode == MODE_FP64) return static_cast<size_t>(sh.warps) * kWarpStage;
+    if (mode == MODE_FP64) return batch64_smem(sh.warps);
     if (sh.r == 0) return static_cast<size_t>(sh.warps) * kSymWarpSmem;
     const size_t bt = 32 * static_cast<size_t>(sh.warps);
     const int len = sh.warps == 4 ? (sh.r == 2 ? block_stage_len<128, 2>() : block_stage_len<128, 1>())
@@ -1010,7 +942,10 @@ static size_t shape_smem(int mode, const BatchShape &sh) {
 
 template <int TENSOR>
 static void *batched_fn_t(int mode, const BatchShape &sh) {
-    if (mode == MODE_FP64) return reinterpret_cast<void *>(&batched_kernel<TENSOR>);
+    if (mode == MODE_FP64)
+        return sh.warps == 4 ? reinterpret_cast<void *>(&batched64_kernel<TENSOR, 4>)
+                             : (sh.warps == 8 ? reinterpret_cast<void *>(&batched64_kernel<TENSOR, 8>)
+                                              : reinterpret_cast<void *>(&batched64_kernel<TENSOR, 16>));
     if (sh.r == 0) return reinterpret_cast<void *>(&batched_sym_kernel<TENSOR>);
     if (sh.r == 2)
         return sh.warps == 4 ? reinterpret_cast<void *>(&batched_blocks_kernel<TENSOR, 128, 2>)
@@ -1245,6 +1180,9 @@ sd_status sd_batch_create(const sd_config *cfg, const int32_t *offsets, int32_t 
     pc.c1_d = 0.75 * a;
     pc.c3_d = 0.5 * a * a * a;
     pc.m3c3_d = -1.5 * a * a * a;
+    pc.k_d = pc.c3_d / pc.c1_d;
+    pc.m3k_d = -3.0 * pc.c3_d / pc.c1_d;
+    pc.invc1_d = 1.0 / pc.c1_d;
     pc.r2min_f = static_cast<float>(pc.r2min_d);
     pc.c1_f = static_cast<float>(pc.c1_d);
     pc.c3_f = static_cast<float>(pc.c3_d);
@@ -1357,8 +1295,9 @@ sd_status sd_batch_create(const sd_config *cfg, const int32_t *offsets, int32_t 
     // thread x resident CTAs per SM
     for (int r : {1, 2, 0}) {
         if (r != 1 && b->mode != MODE_FP32C) continue;
-        for (int w : {4, 8}) {
+        for (int w : {4, 8, 16}) {
             if (r == 0 && w != 4) continue;   // symmetric kernel: 4 warps (tasks) per CTA
+            if (w == 16 && b->mode != MODE_FP64) continue;
             const BatchShape sh1{w, 1, r};
             void *fn = batched_fn(b->tensor, b->mode, sh1);
             const size_t smem = shape_smem(b->mode, sh1);

@@ -31,6 +31,7 @@ struct PairConst {
     float r2min_f, c1_f, c3_f, m3c3_f;   // (2a)^2, 3a/4, a^3/2, -3a^3/2
     double r2min_d, c1_d, c3_d, m3c3_d;
     double a, two_a, mu0;
+    double k_d, m3k_d, invc1_d;          // c3 / c1, -3 c3 / c1, 1 / c1 (profile64)
     // periodic box, nearest image only (Sec. 3.1 footnote): side L_d, 1/L_d; both 0
     // in a dimension without periodicity (the minimum image is then the identity)
     float Lf[3], invLf[3];
@@ -337,6 +338,24 @@ __device__ __forceinline__ void pair_sym_f64(double xi, double yi, double zi, do
     by = __fma_rn(u, dy, __fma_rn(A, gy, by));
     bz = __fma_rn(u, dz, __fma_rn(A, gz, bz));
 }
+
+// A / c1 and B / c1 of the Rotne-Prager / Oseen form in FP64 (the sums are multiplied by c1
+// once per particle): 1/r + k/r^3 and 1/r^3 - 3k/r^5 with k = c3 / c1, nine FP64 operations
+// with the root (Oseen: six) and no conversions.
+template <int TENSOR>
+__device__ __forceinline__ void profile64(double r2, const PairConst &c, double &A, double &B) {
+    const double ri = rsqrt_int64(r2), ri2 = __dmul_rn(ri, ri), ri3 = __dmul_rn(ri, ri2);
+    if (TENSOR == T_OSEEN) {
+        A = ri;
+        B = ri3;
+    } else {
+        A = __fma_rn(c.k_d, ri3, ri);
+        B = __dmul_rn(ri2, __fma_rn(c.m3k_d, ri3, ri));
+    }
+}
+
+// x < y for non-negative FP64 values, in integer operations.
+__device__ __forceinline__ bool less_pos64(double x, double y) { return __double_as_longlong(x) < __double_as_longlong(y); }
 
 // ---------------------------------------------------------------- exact FP64 profile
 

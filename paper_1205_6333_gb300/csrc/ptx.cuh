@@ -84,4 +84,29 @@ __device__ __forceinline__ double rsqrt_nr64(double x) {
     return fma(y0 * e, fma(0.375, e, 0.5), y0);
 }
 
+// The same root for the FP64-bound pair loops: GB300 issues two FP64 operations a clock and
+// SM, conversions between FP32 and FP64 among them, and integer operations at 32 times that
+// rate.  So the seed's argument is x's upper 24 significant bits put together with integer
+// operations (relative error below 2^-23: e stays below 2^-21 and the truncated e^3 term
+// below 2^-64), its widening too, and the constants 1/2 and 3/8 are folded into y0 outside
+// the FP64 pipe (y0 / 2 exactly, by the exponent; 3 y0 / 8 rounded in FP32, which e^2 makes
+// a relative 2^-66): four FP64 operations instead of five and two conversions.  x beyond
+// the FP32 range gives 0, as a seed of rsqrt(inf) does.
+__device__ __forceinline__ double widen_pos(float f) {   // a positive normal FP32 value, exactly
+    const unsigned b = __float_as_uint(f);
+    return __hiloint2double(static_cast<int>((b >> 3) + 0x38000000u), static_cast<int>(b << 29));
+}
+__device__ __forceinline__ double rsqrt_int64(double x) {
+    const int hi = __double2hiint(x);
+    const unsigned lo = static_cast<unsigned>(__double2loint(x));
+    const unsigned fb = (static_cast<unsigned>(hi - 0x38000000) << 3) | (lo >> 29);
+    const float y = rsqrt_sfu(__uint_as_float(fb));
+    const bool far = hi >= 0x47f00000;   // x >= 2^128
+    const double y0 = far ? 0.0 : widen_pos(y);
+    const double half = far ? 0.0 : __hiloint2double(__double2hiint(y0) - 0x00100000, __double2loint(y0));
+    const double k = far ? 0.0 : widen_pos(__fmul_rn(0.375f, y));
+    const double e = __fma_rn(-__dmul_rn(x, y0), y0, 1.0);
+    return __fma_rn(__fma_rn(k, e, half), e, y0);
+}
+
 }  // namespace sd
