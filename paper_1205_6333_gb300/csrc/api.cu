@@ -131,30 +131,25 @@ static sd_status launch_check(cudaError_t e, const char *what) {
 
 // ---------------------------------------------------------------- one Euler step
 
-// A Verlet step (constant forces).  The check kernel writes the mirror, the rebuild
-// decision and the clamp flag.  Then two branches run side by side: the all-pairs
-// kernel on st, and on the side stream the rebuild kernels (cell list and
-// xref = x_in; the candidate list within r_near + skin, each particle's run sorted by
-// partner), which read the decision and return at once when no rebuild is due,
-// followed by the FP64 terms of the listed pairs.  The Euler epilogue joins them.
+// A Verlet step.  The check kernel writes the mirror, the rebuild request and the clamp
+// flag.  Then two branches run side by side: the all-pairs kernel on st, and on the side
+// stream the rebuild (cell list and xref = x_in; the candidate list within r_near + skin,
+// each particle's run sorted by partner), whose kernels return at once when none is due,
+// followed by the FP64 terms of the listed pairs.  The Euler epilogue joins them.  With soft
+// repulsion or lubrication the forces need the list, so the rebuild and the forces come first.
 // Neither branch writes what the other reads.  A fresh and a reused list give the
 // same result bit for bit: each particle's list is sorted by partner and entries
 // beyond r_near add exact zeros.
 static cudaError_t launch_verlet_step(sd_handle *h, cudaStream_t st, double dt, const double *x_in, double *x_out) {
     cudaError_t e = launch_verlet_check(h, st, x_in, h->posm);
-    // with soft repulsion the forces need the list: rebuild (when due) and forces first
-    cudaStream_t rb = h->forces_const ? h->side : st;
     if (!h->forces_const) {
-        if (e == cudaSuccess) e = launch_build_cells(h, st, x_in, h->posm, h->xref);
-        if (e == cudaSuccess) e = launch_near_collect(h, st, x_in, h->posm.aos, h->F64, h->frcm.aos, true, true);
+        if (e == cudaSuccess) e = launch_verlet_rebuild(h, st, x_in, h->posm);
         if (e == cudaSuccess) e = launch_forces_list(h, st, x_in);
     }
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, st);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->side, h->ev_fork, 0);
-    if (h->forces_const && e == cudaSuccess) e = launch_build_cells(h, rb, x_in, h->posm, h->xref);
     prof_begin(h, SD_KERNEL_NEAR, h->side);
-    if (h->forces_const && e == cudaSuccess)
-        e = launch_near_collect(h, rb, x_in, h->posm.aos, h->F64, h->frcm.aos, true, true);
+    if (h->forces_const && e == cudaSuccess) e = launch_verlet_rebuild(h, h->side, x_in, h->posm);
     if (e == cudaSuccess) e = launch_near_pairs(h, h->side, x_in, h->posm.aos, h->F64, h->frcm.aos, true);
     prof_end(h, SD_KERNEL_NEAR, h->side);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_join, h->side);
@@ -172,13 +167,7 @@ static bool use_small(const sd_handle *h) { return h->small.on && !h->inject_sta
 
 // The Verlet steps' list around the positions x64[cur].
 static sd_status build_list(sd_handle *h) {
-    SD_CUDA(cudaMemsetAsync(h->d_vl, 0, sizeof(int), h->stream));
-    SD_CUDA(cudaMemsetAsync(h->d_vl, 1, 1, h->stream));   // a rebuild request (bit 2 clear)
-    const double *x = h->x64[h->cur];
-    sd_status s = launch_check(launch_build_cells(h, h->stream, x, h->posm, h->xref), "neighbour list");
-    if (s == SD_OK)
-        s = launch_check(launch_near_collect(h, h->stream, x, h->posm.aos, h->F64, h->frcm.aos, true, true),
-                         "neighbour list");
+    sd_status s = launch_check(launch_verlet_rebuild(h, h->stream, h->x64[h->cur], h->posm, true), "neighbour list");
     h->list_set = s == SD_OK;
     return s;
 }
@@ -546,9 +535,8 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
     int H = 1024;
     while (H < 2 * h->n) H <<= 1;
     c.H = H;
-    c.nblk = (H + 16383) / 16384;   // scan blocks of 16,384 buckets (cells.cu)
     ok = dalloc_t(h, c.cell, n3 / 3) && dalloc_t(h, c.key, n3 / 3) && dalloc_t(h, c.cnt, H) &&
-         dalloc_t(h, c.start, H + 1) && dalloc_t(h, c.bsum, c.nblk) &&
+         dalloc_t(h, c.start, H + 1) && dalloc_t(h, c.bsum, (H + 4095) / 4096) &&
          dalloc_t(h, c.sorted, n3 / 3);
     if (!ok) return fail(SD_ERR_OOM, "device allocation of the cell list");
 
@@ -663,14 +651,11 @@ sd_status sd_set_positions(sd_handle *h, const double *xyz, int on_device) {
         sd_status s = launch_check(launch_stage_pos(h, h->stream, h->x64[h->cur], h->posm), "stage positions");
         if (s != SD_OK) return s;
         // new positions: the previous step's velocities no longer apply (lubrication),
-        // and the steps' neighbour list is built afresh around them, so that a
-        // trajectory resumed from positions read back continues bit for bit
+        // and the first step builds the steps' neighbour list afresh around them, so that a
+        // trajectory resumed from positions read back continues bit for bit (a product
+        // needs no such list: built here, it cost every moved product 35 us)
         if (h->vlag) SD_CUDA(cudaMemsetAsync(h->vlag, 0, 3 * sizeof(double) * h->n, h->stream));
         h->list_set = false;
-        if (h->verlet && !use_small(h)) {   // (the small path needs no list)
-            s = build_list(h);
-            if (s != SD_OK) return s;
-        }
     }
     h->pos_set = true;
     h->cells_valid = false;
@@ -726,7 +711,21 @@ static sd_status ensure_cells(sd_handle *h) {
     if (h->cells_valid) return SD_OK;
     sd_status s = launch_check(launch_build_cells(h, h->stream, h->x64[h->cur], h->posm), "cell list");
     if (s == SD_OK) h->cells_valid = true;
+    h->near_valid = false;   // (a cell-list build empties the candidate list)
     return s;
+}
+
+// The near pass's candidate list at the current positions, with the cell list and the mirror
+// if they are not there yet.  (The VJP needs the list alone, so it keeps the one that is there;
+// for the product the pass also corrects, in place, the particles that a full list left out.)
+static cudaError_t near_list(sd_handle *h, bool vjp) {
+    const double *x = h->x64[h->cur];
+    if (h->cells_valid && vjp && h->near_valid) return cudaSuccess;
+    h->near_valid = true;
+    if (h->cells_valid) return launch_near_collect(h, h->stream, x, h->posm.aos, h->Fa64, h->frcam.aos, false);
+    const cudaError_t e = launch_near_lists(h, h->stream, x, h->posm, h->Fa64, h->frcam.aos);
+    h->cells_valid = e == cudaSuccess;
+    return e;
 }
 
 // The tile window of the rows [row0, row1): whole i-blocks of the directed kernel.
@@ -773,9 +772,9 @@ static sd_status apply_rows(sd_handle *h, const void *F, void *V, int dtype, int
         return sync_check(h);
     }
     sd_status s = launch_check(launch_stage_forces(h, h->stream, Fd, dtype, 0, h->Fa64, h->frcam), "stage F");
-    if (s == SD_OK) s = ensure_cells(h);
+    if (s == SD_OK) s = launch_check(near_list(h, false), "near pass");
     if (s == SD_OK)
-        s = launch_check(launch_near(h, h->stream, h->x64[h->cur], h->posm.aos, h->Fa64, h->frcam.aos), "near pass");
+        s = launch_check(launch_near_pairs(h, h->stream, h->x64[h->cur], h->posm.aos, h->Fa64, h->frcam.aos), "near pass");
     if (s == SD_OK)
         s = launch_check(launch_dense(h, h->stream, h->posm, h->frcam, h->part, all ? nullptr : &w), "dense kernel");
     if (s == SD_OK)

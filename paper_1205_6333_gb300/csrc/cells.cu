@@ -9,6 +9,7 @@
 // so unbounded domains need no bounding box.  Build = count, exclusive scan,
 // scatter, and an insertion sort of each bucket by particle index (makes every
 // neighbour walk, hence every FP64 near-pair sum, independent of atomics order).
+#include <algorithm>
 #include <type_traits>
 
 #include "neighbours.cuh"
@@ -16,37 +17,6 @@
 namespace sd {
 
 // ---------------------------------------------------------------- staging
-
-// Entry i of a mirror: (x, y, z, 0) in the AoS array and, if present, the SoA copy.
-template <typename V4>
-__device__ __forceinline__ void put_mirror(V4 *aos, float *soa, int npad, int i, double x, double y, double z) {
-    V4 v;
-    v.x = x;
-    v.y = y;
-    v.z = z;
-    v.w = 0;
-    aos[i] = v;
-    if (soa) {
-        soa[i] = static_cast<float>(x);
-        soa[npad + i] = static_cast<float>(y);
-        soa[2 * static_cast<size_t>(npad) + i] = static_cast<float>(z);
-    }
-}
-
-// u wrapped into [0, L) in a periodic dimension (L > 0), unchanged otherwise.
-__device__ __forceinline__ double wrap_box(double u, double L, double invL) {
-    return L > 0.0 ? u - L * floor(u * invL) : u;
-}
-
-// Mirror entry of a position: relative to particle 0 (only differences enter the
-// pair terms, and small coordinates keep FP32 separations accurate), wrapped into
-// the box in periodic dimensions (the pair terms take the nearest image).
-template <typename V4>
-__device__ __forceinline__ void put_pos_mirror(V4 *m, float *soa, int npad, int i, const double *x, const Box &b) {
-    const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-    put_mirror(m, soa, npad, i, wrap_box(px - x[0], b.L[0], b.invL[0]), wrap_box(py - x[1], b.L[1], b.invL[1]),
-               wrap_box(pz - x[2], b.L[2], b.invL[2]));
-}
 
 template <typename V4>
 __global__ void stage_pos_kernel(const double *__restrict__ x, V4 *__restrict__ m, float *__restrict__ soa, int n,
@@ -87,41 +57,41 @@ cudaError_t launch_stage_pos(sd_handle *h, cudaStream_t st, const double *x64, M
 //     positions never set), overflowed (its particles corrected in place), or a
 //     displacement of skin / 2 or more.  (The list is the steps' own, built when the
 //     positions are set and by the steps' rebuilds; no other pass touches it.)
+// A thread takes particles and listed pairs in turn over a grid that reaches every SM: one
+// thread walking a particle's run, in CTAs of 256, took 12 us (N = 4,096) to 17 us (4,913
+// on a lattice); now 8 and 9 us, cold caches.
 template <typename V4>
-__global__ void verlet_check_kernel(const double *__restrict__ x, const double *__restrict__ xref, int n, int npad,
-                                    Box b, double quarter_skin2, double half_skin2, double rsafe2,
-                                    V4 *__restrict__ m, float *__restrict__ soa, int *flag, int *vl,
-                                    const unsigned long long *near_n, int cap, const int2 *__restrict__ ent,
-                                    const int *__restrict__ noff, const int *__restrict__ ncnt, int *err) {
-    __shared__ int s_invalid;
-    if (threadIdx.x == 0) s_invalid = (vl[0] & 2) != 0;
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int bits = s_invalid ? 3 : 0;   // 1: rebuild; 2: clamp every tile
-    if (i < n) {
-        const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-        if (!isfinite(px) || !isfinite(py) || !isfinite(pz)) atomicOr(err, DEV_ERR_NONFINITE);
-        put_pos_mirror(m, soa, npad, i, x, b);
-        const double ux = (px - xref[3 * i]) - (x[0] - xref[0]);
-        const double uy = (py - xref[3 * i + 1]) - (x[1] - xref[1]);
-        const double uz = (pz - xref[3 * i + 2]) - (x[2] - xref[2]);
-        const double u2 = ux * ux + uy * uy + uz * uz;
-        if (!(u2 < quarter_skin2)) bits |= 1;   // (also NaN)
-        if (!(u2 < half_skin2)) bits |= 3;
-        if (i == 0 && *near_n > static_cast<unsigned long long>(cap)) bits |= 3;
-        if (!(bits & 2)) {   // the list is complete around i: its pairs closer than r_safe
-            const int c = ncnt[i];
-            if (c < 0) {
-                bits |= 3;
-            } else {
-                const long long e0 = dbg_index(noff[i], static_cast<long long>(cap) - c + 1, err);
-                for (int k = 0; k < c; ++k) {
-                    const int j = static_cast<int>(dbg_index(ent[e0 + k].y, n, err));
-                    double dx = px - x[3 * j], dy = py - x[3 * j + 1], dz = pz - x[3 * j + 2];
-                    box_image(b, dx, dy, dz);
-                    if (dx * dx + dy * dy + dz * dz < rsafe2) bits |= 2;
-                }
-            }
+__global__ void __launch_bounds__(128) verlet_check_kernel(const double *__restrict__ x, const double *__restrict__ xref,
+                                                           int n, int npad, Box b, double quarter_skin2,
+                                                           double half_skin2, double rsafe2, V4 *__restrict__ m,
+                                                           float *__restrict__ soa, int *flag, int *vl,
+                                                           const unsigned long long *near_n, int cap,
+                                                           const int2 *__restrict__ ent, int *err) {
+    const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x,
+                    stride = static_cast<long long>(gridDim.x) * blockDim.x;
+    const unsigned long long listed = *near_n;
+    // 1: rebuild; 2: clamp every tile (vl[0] is written below, after every block has read it)
+    int bits = (*static_cast<volatile int *>(vl) & 2) || listed > static_cast<unsigned long long>(cap) ? 3 : 0;
+    const long long work = n + (bits ? 0 : static_cast<long long>(listed));   // (a raised clamp bit needs no pairs)
+    for (long long q = gt; q < work; q += stride) {
+        if (q < n) {
+            const long long i = q;
+            const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
+            if (!isfinite(px) || !isfinite(py) || !isfinite(pz)) atomicOr(err, DEV_ERR_NONFINITE);
+            put_pos_mirror(m, soa, npad, static_cast<int>(i), x, b);
+            const double ux = (px - xref[3 * i]) - (x[0] - xref[0]);
+            const double uy = (py - xref[3 * i + 1]) - (x[1] - xref[1]);
+            const double uz = (pz - xref[3 * i + 2]) - (x[2] - xref[2]);
+            const double u2 = ux * ux + uy * uy + uz * uz;
+            if (!(u2 < quarter_skin2)) bits |= 1;   // (also NaN)
+            if (!(u2 < half_skin2)) bits |= 3;
+        } else {
+            const int2 p = ent[q - n];
+            const int i = static_cast<int>(dbg_index(p.x, n, err)), j = static_cast<int>(dbg_index(p.y, n, err));
+            if (i > j) continue;   // (both orders are listed)
+            double dx = x[3 * i] - x[3 * j], dy = x[3 * i + 1] - x[3 * j + 1], dz = x[3 * i + 2] - x[3 * j + 2];
+            box_image(b, dx, dy, dz);
+            if (dx * dx + dy * dy + dz * dz < rsafe2) bits |= 2;
         }
     }
     const int any = (__syncthreads_or(bits & 1) ? 1 : 0) | (__syncthreads_or(bits & 2) ? 2 : 0);
@@ -141,31 +111,39 @@ __global__ void verlet_check_kernel(const double *__restrict__ x, const double *
 
 cudaError_t launch_verlet_check(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm) {
     if (h->n == 0) return cudaSuccess;
-    const int nb = (h->n + 255) / 256;
+    const int nb = static_cast<int>(std::min<long long>((static_cast<long long>(h->n) * 4 + 127) / 128, 4LL * h->num_sms));
     const double hs2 = 0.25 * h->skin * h->skin, qs2 = 0.0625 * h->skin * h->skin;
     const double rs2 = kRSafe * kRSafe * h->pc.a * h->pc.a;
     prof_begin(h, SD_KERNEL_CELLS, st);
     if (h->mode == MODE_FP64)
-        verlet_check_kernel<dbl4><<<nb, 256, 0, st>>>(x64, h->xref, h->n, h->npad, h->cl.box, qs2, hs2, rs2,
+        verlet_check_kernel<dbl4><<<nb, 128, 0, st>>>(x64, h->xref, h->n, h->npad, h->cl.box, qs2, hs2, rs2,
                                                       static_cast<dbl4 *>(posm.aos), posm.soa, h->d_flag, h->d_vl,
-                                                      h->vn, h->near_cap, h->vent, h->voff, h->vcnt, h->d_err);
+                                                      h->vn, h->near_cap, h->vent, h->d_err);
     else
-        verlet_check_kernel<float4><<<nb, 256, 0, st>>>(x64, h->xref, h->n, h->npad, h->cl.box, qs2, hs2, rs2,
-                                                        static_cast<float4 *>(posm.aos), posm.soa, h->d_flag,
-                                                        h->d_vl, h->vn, h->near_cap, h->vent, h->voff, h->vcnt,
-                                                        h->d_err);
+        verlet_check_kernel<float4><<<nb, 128, 0, st>>>(x64, h->xref, h->n, h->npad, h->cl.box, qs2, hs2, rs2,
+                                                        static_cast<float4 *>(posm.aos), posm.soa, h->d_flag, h->d_vl,
+                                                        h->vn, h->near_cap, h->vent, h->d_err);
     prof_end(h, SD_KERNEL_CELLS, st);
     ++h->launches;
     return cudaGetLastError();
 }
 
 // dst64 = src (+ fext + gravity when add_ext) and its mirror; src is n x 3 float or double.
+// A second array (src2, without fext) rides along as the grid's second row.
 template <typename V4, typename Src>
 __global__ void stage_forces_kernel(const Src *__restrict__ src, const double *__restrict__ fext, double gx,
                                     double gy, double gz, double *__restrict__ dst, V4 *__restrict__ m,
-                                    float *__restrict__ soa, int n, int npad, int *err) {
+                                    float *__restrict__ soa, const Src *__restrict__ src2, double *__restrict__ dst2,
+                                    V4 *__restrict__ m2, float *__restrict__ soa2, int n, int npad, int *err) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    if (blockIdx.y) {
+        src = src2;
+        fext = nullptr;
+        dst = dst2;
+        m = m2;
+        soa = soa2;
+    }
     double f[3];
     for (int d = 0; d < 3; ++d) f[d] = src ? static_cast<double>(src[3 * i + d]) : 0.0;
     if (fext) {
@@ -182,25 +160,27 @@ __global__ void stage_forces_kernel(const Src *__restrict__ src, const double *_
 
 template <typename V4, typename Src>
 static void stage_forces_launch(sd_handle *h, cudaStream_t st, const void *src, const double *fe, double *dst64,
-                                Mirror dstm) {
-    const int nb = (h->n + 255) / 256;
+                                Mirror dstm, const void *src2, double *dst2, Mirror dstm2) {
+    const dim3 nb((h->n + 255) / 256, src2 ? 2 : 1);
     const double *g = h->cfg.gravity;
     stage_forces_kernel<V4, Src><<<nb, 256, 0, st>>>(static_cast<const Src *>(src), fe, g[0], g[1], g[2], dst64,
-                                                     static_cast<V4 *>(dstm.aos), dstm.soa, h->n, h->npad, h->d_err);
+                                                     static_cast<V4 *>(dstm.aos), dstm.soa,
+                                                     static_cast<const Src *>(src2), dst2, static_cast<V4 *>(dstm2.aos),
+                                                     dstm2.soa, h->n, h->npad, h->d_err);
 }
 
 // src_dtype: SD_DTYPE_F32 / SD_DTYPE_F64 (src may be NULL = zeros); add_ext: add
 // the handle's F_ext and gravity.
 cudaError_t launch_stage_forces(sd_handle *h, cudaStream_t st, const void *src, int src_dtype, int add_ext,
-                                double *dst64, Mirror dstm) {
+                                double *dst64, Mirror dstm, const void *src2, double *dst2, Mirror dstm2) {
     if (h->n == 0) return cudaSuccess;
     const double *fe = add_ext ? h->fext64 : nullptr;
     if (h->mode == MODE_FP64) {
-        if (src_dtype == SD_DTYPE_F32) stage_forces_launch<dbl4, float>(h, st, src, fe, dst64, dstm);
-        else stage_forces_launch<dbl4, double>(h, st, src, fe, dst64, dstm);
+        if (src_dtype == SD_DTYPE_F32) stage_forces_launch<dbl4, float>(h, st, src, fe, dst64, dstm, src2, dst2, dstm2);
+        else stage_forces_launch<dbl4, double>(h, st, src, fe, dst64, dstm, src2, dst2, dstm2);
     } else {
-        if (src_dtype == SD_DTYPE_F32) stage_forces_launch<float4, float>(h, st, src, fe, dst64, dstm);
-        else stage_forces_launch<float4, double>(h, st, src, fe, dst64, dstm);
+        if (src_dtype == SD_DTYPE_F32) stage_forces_launch<float4, float>(h, st, src, fe, dst64, dstm, src2, dst2, dstm2);
+        else stage_forces_launch<float4, double>(h, st, src, fe, dst64, dstm, src2, dst2, dstm2);
     }
     ++h->launches;
     return cudaGetLastError();
@@ -231,40 +211,23 @@ cudaError_t launch_pad_mirror(sd_handle *h, cudaStream_t st, Mirror m) {
 
 // ---------------------------------------------------------------- cell list
 
-__device__ __forceinline__ int cell_coord(double x, double inv_h) {
-    double c = floor(x * inv_h);
-    c = fmin(fmax(c, -1.0e9), 1.0e9);  // keep the integer in range for absurd coordinates
-    return static_cast<int>(c);
-}
-
-// Cell coordinate in dimension d: nc[d] cells over [0, L) of the wrapped coordinate
-// in a periodic dimension, cells of side h otherwise.
-__device__ __forceinline__ int cell_coord_d(const CellList &c, int d, double x) {
-    const int nc = c.nc[d];
-    if (nc <= 0) return cell_coord(x, c.inv_h);
-    const int k = static_cast<int>(floor(wrap_box(x, c.box.L[d], c.box.invL[d]) * c.box.invL[d] * nc));
-    return k < 0 ? 0 : (k >= nc ? nc - 1 : k);
-}
-
 // Bins particle i and writes its mirror (position relative to particle 0, in the
 // dense kernels' precision), so the mirror is a pure function of the FP64 state.  A
-// Verlet list build (xref given) records the positions in xref instead and leaves
+// Verlet list's build (xref given) records the positions in xref instead and leaves
 // the mirror and the clamp flag to the step's check kernel.
 template <typename V4>
-__global__ void cells_hash_kernel(const double *__restrict__ x, int n, CellList c, int4 *__restrict__ cell,
-                                  uint32_t *__restrict__ key, int *__restrict__ cnt, V4 *__restrict__ m,
+__global__ void cells_hash_kernel(const double *__restrict__ x, int n, CellList c, V4 *__restrict__ m,
                                   float *__restrict__ soa, int npad, int *flag, unsigned long long *near_n,
-                                  double *__restrict__ xref, const int *gate, int *err) {
-    if (gate && *gate == 0) return;   // a Verlet step without a rebuild request
+                                  double *__restrict__ xref, int *vl, int *err) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (i == 0) {
-        *near_n = 0;                // the near pass fills its candidate list from the start
-        if (!xref) *flag = 0;       // ... and raises the flag again if needed
+        *near_n = 0;            // the near pass fills its candidate list from the start
+        if (xref) vl[0] = 0;    // (there is a list)
+        else *flag = 0;         // ... and raises the flag again if needed
     }
-    const int H = c.H;
     const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-    if (xref) {   // a Verlet step's rebuild: the flag and the mirror are its check kernel's
+    if (xref) {
         xref[3 * i] = px;
         xref[3 * i + 1] = py;
         xref[3 * i + 2] = pz;
@@ -272,62 +235,19 @@ __global__ void cells_hash_kernel(const double *__restrict__ x, int n, CellList 
         if (!isfinite(px) || !isfinite(py) || !isfinite(pz)) atomicOr(err, DEV_ERR_NONFINITE);
         put_pos_mirror(m, soa, npad, i, x, c.box);
     }
-    const int cx = cell_coord_d(c, 0, px);
-    const int cy = cell_coord_d(c, 1, py);
-    const int cz = cell_coord_d(c, 2, pz);
-    cell[i] = make_int4(cx, cy, cz, 0);
-    const uint32_t k = cell_hash(cx, cy, cz, H);
-    key[i] = k;
-    atomicAdd(&cnt[k], 1);
+    bin_particle(c, i, px, py, pz);
 }
 
 constexpr int kScanThreads = 1024;
-constexpr int kScanPer = 16;
 constexpr int kScanBlock = kScanThreads * kScanPer;   // buckets one scan block covers (one kernel up to this)
 
-// Exclusive scan of kScanPer values per thread across a block; returns the
-// block total.  Warp shuffles within warps, shared memory across warps.
-__device__ __forceinline__ int block_exclusive_scan(int v[kScanPer], int *s_warp) {
-    int tsum = 0;
-    for (int k = 0; k < kScanPer; ++k) {
-        const int t = v[k];
-        v[k] = tsum;
-        tsum += t;
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int incl = tsum;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        int w = (lane < kScanThreads / 32) ? s_warp[lane] : 0;
-        int wi = w;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += y;
-        }
-        s_warp[lane] = wi - w;  // exclusive warp offsets
-        if (lane == 31) s_warp[32] = wi;
-    }
-    __syncthreads();
-    const int off = s_warp[wid] + incl - tsum;
-    for (int k = 0; k < kScanPer; ++k) v[k] += off;
-    const int total = s_warp[32];
-    __syncthreads();
-    return total;
-}
-
 __global__ void __launch_bounds__(kScanThreads) scan_blocks_kernel(const int *__restrict__ in, int *__restrict__ out,
-                                                                   int *__restrict__ bsum, int H, const int *gate) {
-    if (gate && *gate == 0) return;
+                                                                   int *__restrict__ bsum, int H) {
     __shared__ int s_warp[33];
     const int base = blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
     int v[kScanPer];
     for (int k = 0; k < kScanPer; ++k) v[k] = (base + k < H) ? in[base + k] : 0;
-    const int total = block_exclusive_scan(v, s_warp);
+    const int total = block_exclusive_scan<kScanThreads>(v, s_warp);
     for (int k = 0; k < kScanPer; ++k)
         if (base + k < H) out[base + k] = v[k];
     if (threadIdx.x == 0) {
@@ -339,15 +259,14 @@ __global__ void __launch_bounds__(kScanThreads) scan_blocks_kernel(const int *__
 // One block: exclusive scan of the block totals in place (nblk <= kScanBlock
 // per pass, looping with a carry), then start[H] = grand total.
 __global__ void __launch_bounds__(kScanThreads) scan_top_kernel(int *__restrict__ bsum, int nblk,
-                                                                int *__restrict__ start, int H, const int *gate) {
-    if (gate && *gate == 0) return;
+                                                                int *__restrict__ start, int H) {
     __shared__ int s_warp[33];
     int carry = 0;
     for (int b0 = 0; b0 < nblk; b0 += kScanBlock) {
         const int base = b0 + threadIdx.x * kScanPer;
         int v[kScanPer];
         for (int k = 0; k < kScanPer; ++k) v[k] = (base + k < nblk) ? bsum[base + k] : 0;
-        const int total = block_exclusive_scan(v, s_warp);
+        const int total = block_exclusive_scan<kScanThreads>(v, s_warp);
         for (int k = 0; k < kScanPer; ++k)
             if (base + k < nblk) bsum[base + k] = v[k] + carry;
         carry += total;
@@ -355,75 +274,110 @@ __global__ void __launch_bounds__(kScanThreads) scan_top_kernel(int *__restrict_
     if (threadIdx.x == 0) start[H] = carry;
 }
 
-__global__ void scan_add_kernel(int *__restrict__ start, const int *__restrict__ bsum, int H, const int *gate) {
-    if (gate && *gate == 0) return;
+__global__ void scan_add_kernel(int *__restrict__ start, const int *__restrict__ bsum, int H) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < H) start[e] += bsum[e / kScanBlock];
 }
 
-// Each particle takes a place in its bucket by counting the bucket's occupancy
-// down, which leaves every counter at zero for the next build (no memset).
 __global__ void cells_scatter_kernel(const uint32_t *__restrict__ key, int n, const int *__restrict__ start,
-                                     int *__restrict__ cnt, int *__restrict__ sorted, const int *gate, int *err) {
-    if (gate && *gate == 0) return;
+                                     int *__restrict__ cnt, int *__restrict__ sorted, int *err) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const uint32_t k = key[i];
-    const int pos = start[k] + atomicSub(&cnt[k], 1) - 1;
-    if (pos >= start[k] && pos < start[k + 1])   // always, unless a counter was left non-zero
-        sorted[pos] = i;
-    else
-        atomicOr(err, DEV_ERR_BOUNDS);
+    if (i < n) scatter_particle(key, start, cnt, sorted, i, err);
 }
 
-// Sort each bucket by particle index (buckets hold ~1 particle; a bucket larger
-// than 256 -- only possible for unphysically dense input -- stays unsorted, which
-// changes only the FP64 summation order of its near pairs).
-__global__ void cells_sort_kernel(const int *__restrict__ start, int *__restrict__ sorted, int H, const int *gate) {
-    if (gate && *gate == 0) return;
+__global__ void cells_sort_kernel(const int *__restrict__ start, int *__restrict__ sorted, int H) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= H) return;
-    const int s0 = start[b], s1 = start[b + 1];
-    if (s1 - s0 < 2 || s1 - s0 > 256) return;
-    for (int p = s0 + 1; p < s1; ++p) {
-        const int v = sorted[p];
-        int q = p - 1;
-        while (q >= s0 && sorted[q] > v) {
-            sorted[q + 1] = sorted[q];
-            --q;
-        }
-        sorted[q + 1] = v;
-    }
+    if (b < H) sort_bucket(start, sorted, b);
 }
 
 cudaError_t launch_build_cells(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, double *xref) {
     CellList &c = h->cl;
     if (h->n == 0) return cudaSuccess;
-    // a Verlet build runs only when the step's check asked for it: every kernel reads
-    // the request and returns at once without it
-    const int *gate = xref ? h->d_vl : nullptr;
     prof_begin(h, SD_KERNEL_CELLS, st);
     // (the bucket counters are zero: zeroed at creation, counted back to zero by
     // every build's scatter)
     const int nb = (h->n + 255) / 256;
     if (h->mode == MODE_FP64)
-        cells_hash_kernel<dbl4><<<nb, 256, 0, st>>>(x64, h->n, c, c.cell, c.key, c.cnt,
-                                                    static_cast<dbl4 *>(posm.aos), posm.soa, h->npad, h->d_flag,
-                                                    xref ? h->vn : h->near_n, xref, gate, h->d_err);
+        cells_hash_kernel<dbl4><<<nb, 256, 0, st>>>(x64, h->n, c, static_cast<dbl4 *>(posm.aos), posm.soa, h->npad,
+                                                    h->d_flag, xref ? h->vn : h->near_n, xref, h->d_vl, h->d_err);
     else
-        cells_hash_kernel<float4><<<nb, 256, 0, st>>>(x64, h->n, c, c.cell, c.key, c.cnt,
-                                                      static_cast<float4 *>(posm.aos), posm.soa, h->npad,
-                                                      h->d_flag, xref ? h->vn : h->near_n, xref, gate, h->d_err);
-    scan_blocks_kernel<<<c.nblk, kScanThreads, 0, st>>>(c.cnt, c.start, c.bsum, c.H, gate);
-    if (c.nblk > 1) {
-        scan_top_kernel<<<1, kScanThreads, 0, st>>>(c.bsum, c.nblk, c.start, c.H, gate);
-        scan_add_kernel<<<(c.H + 255) / 256, 256, 0, st>>>(c.start, c.bsum, c.H, gate);
+        cells_hash_kernel<float4><<<nb, 256, 0, st>>>(x64, h->n, c, static_cast<float4 *>(posm.aos), posm.soa, h->npad,
+                                                      h->d_flag, xref ? h->vn : h->near_n, xref, h->d_vl, h->d_err);
+    const int nblk = (c.H + kScanBlock - 1) / kScanBlock;
+    scan_blocks_kernel<<<nblk, kScanThreads, 0, st>>>(c.cnt, c.start, c.bsum, c.H);
+    if (nblk > 1) {
+        scan_top_kernel<<<1, kScanThreads, 0, st>>>(c.bsum, nblk, c.start, c.H);
+        scan_add_kernel<<<(c.H + 255) / 256, 256, 0, st>>>(c.start, c.bsum, c.H);
         h->launches += 2;
     }
-    cells_scatter_kernel<<<nb, 256, 0, st>>>(c.key, h->n, c.start, c.cnt, c.sorted, gate, h->d_err);
-    cells_sort_kernel<<<(c.H + 255) / 256, 256, 0, st>>>(c.start, c.sorted, c.H, gate);
+    cells_scatter_kernel<<<nb, 256, 0, st>>>(c.key, h->n, c.start, c.cnt, c.sorted, h->d_err);
+    cells_sort_kernel<<<(c.H + 255) / 256, 256, 0, st>>>(c.start, c.sorted, c.H);
     prof_end(h, SD_KERNEL_CELLS, st);
     h->launches += 4;
+    return cudaGetLastError();
+}
+
+// A Verlet step's rebuild, if its check asked for one, in one launch: bin, scan, scatter and
+// sort by one cluster, its CTAs meeting at the hardware barrier.  Rebuilds are rare, and
+// what counts is the launch that returns at once: as four to six kernels they cost every
+// step 2 to 3 us each.  CTAs of 256, because the launch
+// shares the GPU with the all-pairs kernel: 1,024 threads found room only after it.  (A
+// cooperative kernel over all SMs costs some 20 us as a graph node; a build that is certain
+// to run takes the kernels above, faster from N = 16,384 on and as fast below.)
+constexpr int kClusterCtas = 8, kClusterThreads = 256, kClusterChunk = kClusterThreads * kScanPer;
+
+__device__ __forceinline__ void cells_barrier() {
+    __threadfence();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    __threadfence();
+}
+
+__global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterThreads)
+    cells_rebuild_kernel(const double *__restrict__ x, int n, CellList c, unsigned long long *list_n, double *xref,
+                         const int *vl, int *err) {
+    if ((*vl & 1) == 0) return;   // (uniform over the cluster; vl is the check kernel's)
+    __shared__ int s_warp[33];
+    const int tid = threadIdx.x, gt = blockIdx.x * kClusterThreads + tid, stride = kClusterCtas * kClusterThreads;
+    for (int i = gt; i < n; i += stride) {
+        const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
+        xref[3 * i] = px;
+        xref[3 * i + 1] = py;
+        xref[3 * i + 2] = pz;
+        bin_particle(c, i, px, py, pz);
+    }
+    if (gt == 0) *list_n = 0;
+    cells_barrier();
+    const int nch = (c.H + kClusterChunk - 1) / kClusterChunk;
+    for (int ch = blockIdx.x; ch < nch; ch += kClusterCtas) {   // scan within each chunk
+        const int base = ch * kClusterChunk + tid * kScanPer;
+        int v[kScanPer];
+        for (int k = 0; k < kScanPer; ++k) v[k] = base + k < c.H ? c.cnt[base + k] : 0;
+        const int total = block_exclusive_scan<kClusterThreads>(v, s_warp);
+        for (int k = 0; k < kScanPer; ++k)
+            if (base + k < c.H) c.start[base + k] = v[k];
+        if (tid == 0) {
+            c.bsum[ch] = total;
+            if (ch == nch - 1) c.start[c.H] = n;   // every particle is in one bucket
+        }
+    }
+    cells_barrier();
+    if (nch > 1) {
+        for (int ch = blockIdx.x; ch < nch; ch += kClusterCtas) {   // ... and the chunks before it
+            int sum = 0;
+            for (int k = 0; k < ch; ++k) sum += c.bsum[k];
+            for (int k = tid; k < kClusterChunk && ch * kClusterChunk + k < c.H; k += kClusterThreads)
+                c.start[ch * kClusterChunk + k] += sum;
+        }
+        cells_barrier();
+    }
+    for (int i = gt; i < n; i += stride) scatter_particle(c.key, c.start, c.cnt, c.sorted, i, err);
+    cells_barrier();
+    for (int b = gt; b < c.H; b += stride) sort_bucket(c.start, c.sorted, b);
+}
+
+cudaError_t launch_rebuild_cells(sd_handle *h, cudaStream_t st, const double *x64) {
+    cells_rebuild_kernel<<<kClusterCtas, kClusterThreads, 0, st>>>(x64, h->n, h->cl, h->vn, h->xref, h->d_vl, h->d_err);
+    ++h->launches;
     return cudaGetLastError();
 }
 
@@ -514,23 +468,36 @@ __global__ void forces_rep_kernel(const double *__restrict__ x, const double *__
 
 // Forces of a Verlet step (Sec. 3.1, step 2) with soft repulsion and/or lubrication:
 // the pairs come from the steps' near-pair list (it holds every pair within the
-// largest cutoff while the list is valid), one thread per particle over its run in
-// ascending partner order, in FP64; the terms are forces_rep_kernel's.  Plus F_ext and
-// gravity.  Writes F64 and the force mirror.
-template <typename V4>
-__global__ void forces_list_kernel(const double *__restrict__ x, const double *__restrict__ fext, double gx,
+// largest cutoff while the list is valid), in FP64; the terms are forces_rep_kernel's.  Plus
+// F_ext and gravity.  Writes F64 and the force mirror.
+// Some 60 FP64 operations a pair, two a clock and SM, so what counts is that every SM and
+// every lane has pairs: in CTAs of 64, L lanes take a particle's run in turn, and its terms
+// are added in ascending partner order (entries beyond the cutoff add zeros wherever they
+// stand in the run).  One thread per particle in CTAs of 128 left most SMs idle at small n
+// (N = 4,913, lubrication: 19 us, with four lanes 13; cold caches); from kForceWideN particles
+// on one lane each fills them, and four cost more in the ordered sum (16,384, repulsion: 16 us
+// against 13).
+constexpr int kForceWideN = 8192;
+template <typename V4, int L>
+__global__ void __launch_bounds__(64) forces_list_kernel(const double *__restrict__ x, const double *__restrict__ fext, double gx,
                                    double gy, double gz, double eps, double rc, double s12,
                                    const double *__restrict__ vlag, double inv_a, double inv_mu0, CellList c,
                                    const int2 *__restrict__ ent, const int *__restrict__ noff,
                                    const int *__restrict__ ncnt, int cap, int n, int npad, double *__restrict__ F,
                                    V4 *__restrict__ m, float *__restrict__ soa, int *err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int i = static_cast<int>(gt / L), sub = static_cast<int>(gt % L);
+    const bool active = i < n;
     const bool rep = eps != 0.0, lub = vlag != nullptr;
     const double rc2 = rep ? rc * rc : 0.0;
     const double rl2 = lub ? 9.0 / (inv_a * inv_a) : 0.0;   // (3a)^2
     const double rmax2 = rc2 > rl2 ? rc2 : rl2;
-    const double xi = x[3 * i], yi = x[3 * i + 1], zi = x[3 * i + 2];
+    double xi = 0.0, yi = 0.0, zi = 0.0;
+    if (active) {
+        xi = x[3 * i];
+        yi = x[3 * i + 1];
+        zi = x[3 * i + 2];
+    }
     double f[3] = {0.0, 0.0, 0.0};
     bool coincident = false;
     auto pair = [&](int j) {
@@ -575,15 +542,26 @@ __global__ void forces_list_kernel(const double *__restrict__ x, const double *_
             }
         }
     };
-    const int cnt = ncnt[i];
+    const int cnt = active ? ncnt[i] : 0;
+    double sum[3] = {0.0, 0.0, 0.0};
     if (cnt < 0) {   // a particle the overflowed list corrects in place: the cell list (rebuilt
                      // every step while the list overflows) gives its pairs
-        for_each_neighbour_part(c, i, c.cell[i], 0, 1, pair);
-    } else {
-        const long long e0 = dbg_index(noff[i], static_cast<long long>(cap) - cnt + 1, err);
-        for (int k = 0; k < cnt; ++k) pair(static_cast<int>(dbg_index(ent[e0 + k].y, n, err)));
+        if (sub == 0) for_each_neighbour_part(c, i, c.cell[i], 0, 1, pair);
+        for (int d = 0; d < 3; ++d) sum[d] = f[d];
     }
-    const double f0 = f[0] + fext[3 * i] + gx, f1 = f[1] + fext[3 * i + 1] + gy, f2v = f[2] + fext[3 * i + 2] + gz;
+    const long long e0 = cnt > 0 ? dbg_index(noff[i], static_cast<long long>(cap) - cnt + 1, err) : 0;
+    const int rounds = __reduce_max_sync(0xffffffffu, (max(cnt, 0) + L - 1) / L);
+    for (int r = 0; r < rounds; ++r) {
+        const int k = r * L + sub;
+        f[0] = f[1] = f[2] = 0.0;
+        if (k < cnt) pair(static_cast<int>(dbg_index(ent[e0 + k].y, n, err)));
+#pragma unroll
+        for (int l = 0; l < L; ++l)
+            for (int d = 0; d < 3; ++d) sum[d] += __shfl_sync(0xffffffffu, f[d], l, L);
+    }
+    coincident = __any_sync(0xffffffffu, coincident);
+    if (!active || sub != 0) return;
+    const double f0 = sum[0] + fext[3 * i] + gx, f1 = sum[1] + fext[3 * i + 1] + gy, f2v = sum[2] + fext[3 * i + 2] + gz;
     if (coincident) atomicOr(err, DEV_ERR_COINCIDENT);
     if (!isfinite(f0) || !isfinite(f1) || !isfinite(f2v)) atomicOr(err, DEV_ERR_NONFINITE);
     F[3 * i] = f0;
@@ -594,22 +572,23 @@ __global__ void forces_list_kernel(const double *__restrict__ x, const double *_
 
 cudaError_t launch_forces_list(sd_handle *h, cudaStream_t st, const double *x64) {
     if (h->n == 0) return cudaSuccess;
-    const int nb = (h->n + 127) / 128;
+    const bool wide = h->n < kForceWideN;
+    const int nb = static_cast<int>((static_cast<long long>(h->n) * (wide ? 4 : 1) + 63) / 64);
     const double *g = h->cfg.gravity;
     const double s12 = pow(2.0 * h->cfg.a, 12.0);
     const double *vlag = h->lub ? h->vlag : nullptr;
     const double inv_a = 1.0 / h->pc.a, inv_mu0 = 1.0 / h->pc.mu0;
     prof_begin(h, SD_KERNEL_FORCES, st);
-    if (h->mode == MODE_FP64)
-        forces_list_kernel<dbl4><<<nb, 128, 0, st>>>(x64, h->fext64, g[0], g[1], g[2], h->cfg.rep_eps, h->rep_rc,
-                                                     s12, vlag, inv_a, inv_mu0, h->cl, h->vent, h->voff, h->vcnt,
-                                                     h->near_cap, h->n, h->npad, h->F64,
-                                                     static_cast<dbl4 *>(h->frcm.aos), h->frcm.soa, h->d_err);
-    else
-        forces_list_kernel<float4><<<nb, 128, 0, st>>>(x64, h->fext64, g[0], g[1], g[2], h->cfg.rep_eps, h->rep_rc,
-                                                       s12, vlag, inv_a, inv_mu0, h->cl, h->vent, h->voff, h->vcnt,
-                                                       h->near_cap, h->n, h->npad, h->F64,
-                                                       static_cast<float4 *>(h->frcm.aos), h->frcm.soa, h->d_err);
+#define SD_FORCES(VV, LL)                                                                                            \
+    forces_list_kernel<VV, LL><<<nb, 64, 0, st>>>(x64, h->fext64, g[0], g[1], g[2], h->cfg.rep_eps, h->rep_rc, s12, vlag, \
+                                                  inv_a, inv_mu0, h->cl, h->vent, h->voff, h->vcnt, h->near_cap, h->n,   \
+                                                  h->npad, h->F64, static_cast<VV *>(h->frcm.aos), h->frcm.soa, h->d_err)
+    if (h->mode == MODE_FP64) {
+        if (wide) SD_FORCES(dbl4, 4); else SD_FORCES(dbl4, 1);
+    } else {
+        if (wide) SD_FORCES(float4, 4); else SD_FORCES(float4, 1);
+    }
+#undef SD_FORCES
     prof_end(h, SD_KERNEL_FORCES, st);
     ++h->launches;
     return cudaGetLastError();

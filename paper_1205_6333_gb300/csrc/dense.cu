@@ -894,6 +894,7 @@ cudaError_t dense_setup(sd_handle *h) {
     const int nreal = std::max(h->n, 1);
     g.nIB = (nreal + g.I - 1) / g.I;
     void *fn = pick_dense(h->tensor, h->mode, h->pc.periodic != 0);
+    const void *chosen = fn;
     const int Jcand[4] = {kJmax, 128, 64, 32};
     int occ = 0;
     for (int ci = 0; ci < 4; ++ci) {
@@ -954,6 +955,7 @@ cudaError_t dense_setup(sd_handle *h) {
             g = s;
             occ = socc;
             h->sym_nt = kB64;
+            chosen = sfn;
         }
     }
     if (h->mode != MODE_FP64 && h->npad % B == 0 && want_sym != SD_DENSE_DIRECTED) {
@@ -979,8 +981,11 @@ cudaError_t dense_setup(sd_handle *h) {
             g = s;
             occ = socc;
             h->sym_nt = NT;
+            chosen = sfn;
         }
     }
+    cudaError_t ea = allow_smem(chosen, h->dense_limit);
+    if (ea != cudaSuccess) return ea;
     int ms = 0;
     for (int ib = 0; ib < g.nIB; ++ib) ms = std::max(ms, geom_last(g, ib) - geom_first(g, ib) + 1);
     g.maxSlots = ms;
@@ -996,17 +1001,18 @@ template <bool PER>
 static void launch_dense_t(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, double *part, const TileWin &w,
                            int grid) {
     const DenseGeom &g = h->geom;
-    const size_t smem = dense_smem(h->mode, g.J);
+    const size_t need = g.sym ? (h->mode == MODE_FP64 ? sym64_smem() : sym_smem(g.I, h->sym_nt)) : dense_smem(h->mode, g.J);
+    const size_t smem = spread_smem(h->num_sms, grid, h->dense_occ, need, h->dense_limit);
     const bool oseen = h->tensor == T_OSEEN;
     if (h->mode == MODE_FP64) {
         const dbl4 *p = static_cast<const dbl4 *>(posm.aos), *f = static_cast<const dbl4 *>(frcm.aos);
         if (g.sym) {
             double *jp = static_cast<double *>(h->jpart);
             if (oseen)
-                dense_sym64_kernel<T_OSEEN, PER><<<grid, kB64, sym64_smem(), st>>>(p, f, part, jp, h->npad, g, h->pc,
+                dense_sym64_kernel<T_OSEEN, PER><<<grid, kB64, smem, st>>>(p, f, part, jp, h->npad, g, h->pc,
                                                                                  h->d_err, dense_wd(h), w.b0);
             else
-                dense_sym64_kernel<T_RP, PER><<<grid, kB64, sym64_smem(), st>>>(p, f, part, jp, h->npad, g, h->pc,
+                dense_sym64_kernel<T_RP, PER><<<grid, kB64, smem, st>>>(p, f, part, jp, h->npad, g, h->pc,
                                                                               h->d_err, dense_wd(h), w.b0);
             return;
         }
@@ -1022,7 +1028,7 @@ static void launch_dense_t(sd_handle *h, cudaStream_t st, Mirror posm, Mirror fr
     const bool comp = h->mode == MODE_FP32C;
     if (g.sym) {
 #define SD_DS(TT, CC, BB, NN)                                                                                  \
-    dense_sym_kernel<TT, CC, PER, BB, NN><<<grid, NN, sym_smem(BB, NN), st>>>(posm.soa, frcm.soa, part,       \
+    dense_sym_kernel<TT, CC, PER, BB, NN><<<grid, NN, smem, st>>>(posm.soa, frcm.soa, part,       \
                                                                               static_cast<float *>(h->jpart), h->npad, \
                                                                               g, c2, h->d_flag, h->d_err, dense_wd(h), \
                                                                               w.b0)

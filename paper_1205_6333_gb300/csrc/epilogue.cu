@@ -23,6 +23,7 @@
 // small separations) or that the clamp altered (r < 2a).
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 #include "neighbours.cuh"
 
 namespace sd {
@@ -107,7 +108,6 @@ struct NearArgs {
     unsigned long long *ent_n;   // entries claimed (zeroed before the collect kernel)
     int *noff, *ncnt; // per particle: first entry and count; ncnt = -1: correction is in near[i]
     int cap;
-    const int *gate;  // Verlet list build: run only when the step's check asked for a rebuild
 };
 
 // The correction of one near pair (FP64 r^2 < r_near^2), added to c6: the exact
@@ -201,12 +201,12 @@ __device__ void near_direct(const NearArgs &a, int i, int sub, bool active) {
 // would).
 constexpr int kNearRegs = 4;   // candidates a lane keeps in registers; more -> second walk
 
-template <int TENSOR, int MODE>
-__global__ void __launch_bounds__(128) near_collect_kernel(NearArgs a) {
-    if (a.gate && *a.gate == 0) return;   // (uniform over the grid)
+// gt: this thread's place among the walk's threads (kWalkLanes per particle); SORT: each
+// particle's run by partner index.  Warp-collective.
+template <int TENSOR, int MODE, bool SORT>
+__device__ __forceinline__ void near_collect(const NearArgs &a, long long gt) {
     using V4 = typename EpiT<MODE>::V4;
     const V4 *pm = static_cast<const V4 *>(a.posm);
-    const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     const int q = static_cast<int>(gt / kWalkLanes), sub = static_cast<int>(gt % kWalkLanes);
     const bool active = q < a.n;
     const int i = active ? a.cl.sorted[q] : 0;
@@ -268,12 +268,12 @@ __global__ void __launch_bounds__(128) near_collect_kernel(NearArgs a) {
         if (active && sub == 0) a.ncnt[i] = -1;
         near_direct<TENSOR, MODE>(a, i, sub, active);
     }
-    // A Verlet list (a.gate set): each particle's run in ascending partner index, so
+    // A Verlet list (SORT): each particle's run in ascending partner index, so
     // that the epilogue adds a particle's near terms in an order that does not depend
     // on when, or from which cell list, the list was built (entries beyond r_near add
     // exact zeros).  The run was written by this warp's lanes of the particle.
     __syncwarp();
-    if (a.gate && fits && active && sub == 0 && pcnt > 1) {
+    if (SORT && fits && active && sub == 0 && pcnt > 1) {
         for (int p = pfirst + 1; p < pfirst + pcnt; ++p) {
             const int2 v = a.ent[p];
             int q = p - 1;
@@ -284,6 +284,13 @@ __global__ void __launch_bounds__(128) near_collect_kernel(NearArgs a) {
             a.ent[q + 1] = v;
         }
     }
+}
+
+// gate: run only when the Verlet step's check asked for a rebuild.
+template <int TENSOR, int MODE, bool SORT>
+__global__ void __launch_bounds__(128) near_collect_kernel(NearArgs a, const int *gate) {
+    if (gate && (*gate & 1) == 0) return;   // (uniform over the grid)
+    near_collect<TENSOR, MODE, SORT>(a, static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x);
 }
 
 // Step 2: one thread per listed pair: the FP64 test r < r_near, the flags, and the
@@ -318,7 +325,11 @@ __global__ void __launch_bounds__(128) near_pair_kernel(NearArgs a) {
 
 template <int TENSOR, int MODE>
 static void near_launch_collect(int nb, cudaStream_t st, const NearArgs &a) {
-    near_collect_kernel<TENSOR, MODE><<<nb, 128, 0, st>>>(a);
+    near_collect_kernel<TENSOR, MODE, false><<<nb, 128, 0, st>>>(a, nullptr);
+}
+template <int TENSOR, int MODE>
+static void near_launch_collect_sorted(std::pair<int, const int *> l, cudaStream_t st, const NearArgs &a) {
+    near_collect_kernel<TENSOR, MODE, true><<<l.first, 128, 0, st>>>(a, l.second);
 }
 template <int TENSOR, int MODE>
 static void near_launch_pairs(int np, cudaStream_t st, const NearArgs &a) {
@@ -348,7 +359,6 @@ static NearArgs near_args(sd_handle *h, const double *x64, const void *posm, con
     a.noff = vlist ? h->voff : h->near_off;
     a.ncnt = vlist ? h->vcnt : h->near_cnt;
     a.cap = h->near_cap;
-    a.gate = nullptr;
     return a;
 }
 
@@ -363,13 +373,9 @@ static NearArgs near_args(sd_handle *h, const double *x64, const void *posm, con
     } while (0)
 
 cudaError_t launch_near_collect(sd_handle *h, cudaStream_t st, const double *x64, const void *posm,
-                                const double *F64, const void *frcm, bool count_zeroed, bool verlet_list) {
+                                       const double *F64, const void *frcm, bool count_zeroed) {
     if (h->n == 0) return cudaSuccess;
-    NearArgs a = near_args(h, x64, posm, F64, frcm, verlet_list ? h->list_cut + h->skin : h->r_near, verlet_list);
-    if (verlet_list) {   // a Verlet step's rebuild: the clamp flag is its check kernel's
-        a.gate = h->d_vl;
-        a.flag = nullptr;
-    }
+    NearArgs a = near_args(h, x64, posm, F64, frcm, h->r_near);
     const int nb = static_cast<int>((static_cast<long long>(h->n) * kWalkLanes + 127) / 128);
     if (!count_zeroed) {
         cudaError_t e = cudaMemsetAsync(a.ent_n, 0, sizeof(*a.ent_n), st);
@@ -380,13 +386,39 @@ cudaError_t launch_near_collect(sd_handle *h, cudaStream_t st, const double *x64
     return cudaGetLastError();
 }
 
+// The Verlet list of the cells (cutoff + skin, sorted runs), behind the gate.
+static cudaError_t launch_verlet_list(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, const int *gate) {
+    NearArgs a = near_args(h, x64, posm.aos, h->F64, h->frcm.aos, h->list_cut + h->skin, true);
+    a.flag = nullptr;   // (the check's)
+    const int nb = static_cast<int>((static_cast<long long>(h->n) * kWalkLanes + 127) / 128);
+    SD_NEAR_DISPATCH(near_launch_collect_sorted, std::make_pair(nb, gate));
+    ++h->launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_verlet_rebuild(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, bool build) {
+    if (h->n == 0) return cudaSuccess;
+    cudaError_t e = build ? launch_build_cells(h, st, x64, posm, h->xref) : launch_rebuild_cells(h, st, x64);
+    if (e == cudaSuccess) e = launch_verlet_list(h, st, x64, posm, build ? nullptr : h->d_vl);
+    return e;
+}
+
+cudaError_t launch_near_lists(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, const double *F64,
+                              const void *frcm) {
+    if (h->n == 0) return cudaSuccess;
+    cudaError_t e = launch_build_cells(h, st, x64, posm);
+    if (e == cudaSuccess) e = launch_near_collect(h, st, x64, posm.aos, F64, frcm, true);
+    return e;
+}
+
 cudaError_t launch_near_pairs(sd_handle *h, cudaStream_t st, const double *x64, const void *posm, const double *F64,
                               const void *frcm, bool verlet_step) {
     if (h->n == 0) return cudaSuccess;
     NearArgs a = near_args(h, x64, posm, F64, frcm, h->r_near, verlet_step);
     if (verlet_step) a.flag = nullptr;   // (the check kernel's; the all-pairs kernel may be reading it)
-    const int np = static_cast<int>(std::min<long long>((static_cast<long long>(a.cap) + 127) / 128,
-                                                        8LL * h->num_sms));
+    // two pairs a particle in one pass, any more in turn (CTAs that find no pair crowd the
+    // all-pairs kernel beside them)
+    const int np = static_cast<int>(std::min<long long>((2LL * h->n + 127) / 128, 8LL * h->num_sms));
     SD_NEAR_DISPATCH(near_launch_pairs, np);
     ++h->launches;
     return cudaGetLastError();
@@ -397,7 +429,7 @@ cudaError_t launch_near(sd_handle *h, cudaStream_t st, const double *x64, const 
                         const void *frcm, bool count_zeroed) {
     if (h->n == 0) return cudaSuccess;
     prof_begin(h, SD_KERNEL_NEAR, st);
-    cudaError_t e = launch_near_collect(h, st, x64, posm, F64, frcm, count_zeroed, false);
+    cudaError_t e = launch_near_collect(h, st, x64, posm, F64, frcm, count_zeroed);
     if (e == cudaSuccess) e = launch_near_pairs(h, st, x64, posm, F64, frcm, false);
     prof_end(h, SD_KERNEL_NEAR, st);
     return e;
@@ -463,11 +495,17 @@ __device__ __forceinline__ int first_row_at(const DenseGeom &g, int ib, long lon
 #ifndef SD_EPI_UNROLL
 #define SD_EPI_UNROLL 2
 #endif
+// Up to SD_EPI_SMALL_N particles the sums are short and the kernel is a chain of dependent
+// loads: eight warps per 32 particles and one particle per lane (more, shorter chains on more
+// SMs), twice the unrolling, and the loads of the tail issued before the sums (16,384: 19.1 ->
+// 17.9 us, cold caches).
+#ifndef SD_EPI_SMALL_N
+#define SD_EPI_SMALL_N 16384
+#endif
 #ifndef SD_EPI_PAIRS
 #define SD_EPI_PAIRS 1
 #endif
 constexpr int kEpiWarps = SD_EPI_WARPS;
-constexpr int kEpiUnroll = SD_EPI_UNROLL;
 constexpr bool kEpiPairs = SD_EPI_PAIRS != 0;   // FP32C: two particles per lane in the sums
 
 // P particles per lane in the sums (P = 2: FP32C without shard shares, row0 even):
@@ -475,17 +513,38 @@ constexpr bool kEpiPairs = SD_EPI_PAIRS != 0;   // FP32C: two particles per lane
 // and their source-side partials as one 8-byte load, so each load instruction
 // carries twice the bytes; every particle's sums take the same operations in the
 // same order as with P = 1.
-template <int TDENSE, int MODE, int OUT, int P>
-__global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
+template <int TDENSE, int MODE, int OUT, int P, int W>
+__global__ void __launch_bounds__(32 * W) epilogue_kernel(EpiArgs a) {
     using V4 = typename EpiT<MODE>::V4;
     constexpr int NP = 32 * P;   // particles per CTA
+    constexpr bool EARLY = W > kEpiWarps;   // the variant of small systems
+    constexpr int U = EARLY ? 4 : SD_EPI_UNROLL;
     static_assert(P == 1 || (P == 2 && MODE == MODE_FP32C), "two particles per lane: FP32C only");
-    __shared__ double s_v[kEpiWarps][3][NP];
-    __shared__ float s_h[kEpiWarps][3][NP], s_l[kEpiWarps][3][NP];
+    __shared__ double s_v[W][3][NP];
+    __shared__ float s_h[W][3][NP], s_l[W][3][NP];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     // CTAs in reverse particle order: the last blocks have the longest source-side
     // columns, so they start first instead of forming the tail
     const int base = a.row0 + (gridDim.x - 1 - blockIdx.x) * NP;
+
+    // what the particle's finishing thread needs besides the sums
+    struct Tail {
+        V4 p, f;
+        double F[3], x[3];
+        int var, cnt, off;
+    } tl;
+    auto load_tail = [&](int i) {
+        tl.p = static_cast<const V4 *>(a.posm)[i];
+        tl.f = static_cast<const V4 *>(a.frcm)[i];
+        for (int d = 0; d < 3; ++d) tl.F[d] = a.F64[3 * i + d];
+        tl.var = (*a.flag) ? 0 : 3;
+        tl.cnt = a.ncnt[i];
+        tl.off = a.noff[i];
+        if constexpr (OUT == OUT_EULER)
+            for (int d = 0; d < 3; ++d) tl.x[d] = a.x64[3 * i + d];
+    };
+    if constexpr (EARLY && OUT != OUT_PART)
+        if (w < P && base + 32 * w + lane < a.row1) load_tail(base + 32 * w + lane);
 
     // This warp's share of the dense sum: the CTA slots of the particle's i-block,
     // then (symmetric kernel) the source-side slots of the tiles (r, ib), r < ib.
@@ -522,39 +581,39 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
             const int J = a.g.J;
             const size_t cs = 3 * static_cast<size_t>(J);
             if constexpr (MODE == MODE_FP32) {
-                for (int s = s0 + w; s < ns; s += kEpiWarps)
+                for (int s = s0 + w; s < ns; s += W)
                     for (int d = 0; d < 3; ++d)
                         hi[0][d] = __fadd_rn(hi[0][d], static_cast<float>(
                                                            a.part[(static_cast<size_t>(s) * 3 + d) * a.npad + i]));
-                for (int r = r0 + w; r < nc; r += kEpiWarps) {
+                for (int r = r0 + w; r < nc; r += W) {
                     const float *src = a.jpart + static_cast<size_t>(geom_rowstart(a.g, r) + (ib - r)) * cs + o;
                     for (int d = 0; d < 3; ++d) hi[0][d] = __fadd_rn(hi[0][d], src[d * J]);
                 }
             } else if constexpr (MODE == MODE_FP64) {
-                for (int s = s0 + w; s < ns; s += kEpiWarps)
+                for (int s = s0 + w; s < ns; s += W)
                     for (int d = 0; d < 3; ++d) v[0][d] += a.part[(static_cast<size_t>(s) * 3 + d) * a.npad + i];
-                for (int r = r0 + w; r < nc; r += kEpiWarps) {
+                for (int r = r0 + w; r < nc; r += W) {
                     const double *src = a.jpart64 + static_cast<size_t>(geom_rowstart(a.g, r) + (ib - r)) * cs + o;
                     for (int d = 0; d < 3; ++d) v[0][d] += src[d * J];
                 }
             } else if constexpr (P == 1) {   // FP32C: each slot is a (hi, lo) float pair
                 const float2 *pp = reinterpret_cast<const float2 *>(a.part);
 #pragma unroll 4
-                for (int s = s0 + w; s < ns; s += kEpiWarps)
+                for (int s = s0 + w; s < ns; s += W)
                     for (int d = 0; d < 3; ++d) {
                         const float2 q = pp[(static_cast<size_t>(s) * 3 + d) * a.npad + i];
                         fold2(hi[0][d], lo[0][d], q.x);
                         lo[0][d] = __fadd_rn(lo[0][d], q.y);
                     }
-#pragma unroll kEpiUnroll
-                for (int r = r0 + w; r < nc; r += kEpiWarps) {
+#pragma unroll U
+                for (int r = r0 + w; r < nc; r += W) {
                     const float *src = a.jpart + static_cast<size_t>(geom_rowstart(a.g, r) + (ib - r)) * cs + o;
                     for (int d = 0; d < 3; ++d) fold2(hi[0][d], lo[0][d], src[d * J]);
                 }
             } else {   // FP32C, two particles: i even, npad, I and J even, so both loads are aligned
                 const float2 *pp = reinterpret_cast<const float2 *>(a.part);
 #pragma unroll 4
-                for (int s = s0 + w; s < ns; s += kEpiWarps)
+                for (int s = s0 + w; s < ns; s += W)
                     for (int d = 0; d < 3; ++d) {
                         const float4 q =
                             *reinterpret_cast<const float4 *>(pp + (static_cast<size_t>(s) * 3 + d) * a.npad + i);
@@ -563,8 +622,8 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
                         fold2(hi[1][d], lo[1][d], q.z);
                         lo[1][d] = __fadd_rn(lo[1][d], q.w);
                     }
-#pragma unroll kEpiUnroll
-                for (int r = r0 + w; r < nc; r += kEpiWarps) {
+#pragma unroll U
+                for (int r = r0 + w; r < nc; r += W) {
                     const float *src = a.jpart + static_cast<size_t>(geom_rowstart(a.g, r) + (ib - r)) * cs + o;
                     for (int d = 0; d < 3; ++d) {
                         const float2 q = *reinterpret_cast<const float2 *>(src + d * J);
@@ -587,18 +646,16 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
     const int j = 32 * w + lane;   // the particle's place in the CTA's sums
     const int i = base + j;
     if (i >= a.row1) return;
-    const V4 *pm = static_cast<const V4 *>(a.posm);
-    const V4 *fm = static_cast<const V4 *>(a.frcm);
     double V[3];
     for (int d = 0; d < 3; ++d) {
         if constexpr (MODE == MODE_FP32) {
             float f = s_h[0][d][j];
-            for (int q = 1; q < kEpiWarps; ++q) f = __fadd_rn(f, s_h[q][d][j]);
+            for (int q = 1; q < W; ++q) f = __fadd_rn(f, s_h[q][d][j]);
             V[d] = f;
         } else {
             double v = s_v[0][d][j];
             float h = s_h[0][d][j], l = s_l[0][d][j];
-            for (int q = 1; q < kEpiWarps; ++q) {
+            for (int q = 1; q < W; ++q) {
                 v += s_v[q][d][j];
                 fold2(h, l, s_h[q][d][j]);
                 l = __fadd_rn(l, s_l[q][d][j]);
@@ -615,22 +672,21 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
     }
     // self term: the tile holding it was clamped; replace by mu_ii / mu0 = I
     {
-        const V4 pi = pm[i];
+        if constexpr (!EARLY) load_tail(i);
         double t[3];
-        dense_term<TDENSE, MODE, true>(pi, pi, fm[i], a.pc, t);
-        for (int d = 0; d < 3; ++d) V[d] += a.F64[3 * i + d] - t[d];
+        dense_term<TDENSE, MODE, true>(tl.p, tl.p, tl.f, a.pc, t);
+        for (int d = 0; d < 3; ++d) V[d] += tl.F[d] - t[d];
     }
     // near pairs: the variant matching the kernel's clamping, from the particle's
     // entries of the candidate list in list order (or from its in-place result)
     {
-        const int var = (*a.flag) ? 0 : 3;
-        const int cnt = a.ncnt[i];
+        const int cnt = tl.cnt;
         if (cnt < 0) {
-            const double *c = a.near + 6 * static_cast<size_t>(i) + var;
+            const double *c = a.near + 6 * static_cast<size_t>(i) + tl.var;
             for (int d = 0; d < 3; ++d) V[d] += c[d];
         } else {
-            const long long e0 = dbg_index(a.noff[i], static_cast<long long>(a.cap) - cnt + 1, a.err);
-            const double *c = a.ent_out + 6 * static_cast<size_t>(e0) + var;
+            const long long e0 = dbg_index(tl.off, static_cast<long long>(a.cap) - cnt + 1, a.err);
+            const double *c = a.ent_out + 6 * static_cast<size_t>(e0) + tl.var;
             for (int k = 0; k < cnt; ++k, c += 6)
                 for (int d = 0; d < 3; ++d) V[d] += c[d];
         }
@@ -648,8 +704,7 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
         o[1] = v1;
         o[2] = v2;
     } else {
-        const double xi = a.x64[3 * i], yi = a.x64[3 * i + 1], zi = a.x64[3 * i + 2];
-        const double nx = xi + a.dt * v0, ny = yi + a.dt * v1, nz = zi + a.dt * v2;
+        const double nx = tl.x[0] + a.dt * v0, ny = tl.x[1] + a.dt * v1, nz = tl.x[2] + a.dt * v2;
         if (a.vlag) {
             a.vlag[3 * i] = v0;
             a.vlag[3 * i + 1] = v1;
@@ -662,29 +717,34 @@ __global__ void __launch_bounds__(32 * kEpiWarps) epilogue_kernel(EpiArgs a) {
     }
 }
 
-template <int TDENSE, int MODE, int P>
+template <int TDENSE, int MODE, int P, int W>
 static void epi_launch(int out, cudaStream_t st, const EpiArgs &a) {
     const int nb = (a.row1 - a.row0 + 32 * P - 1) / (32 * P);
     switch (out) {
-        case OUT_F32: epilogue_kernel<TDENSE, MODE, OUT_F32, P><<<nb, 32 * kEpiWarps, 0, st>>>(a); break;
-        case OUT_F64: epilogue_kernel<TDENSE, MODE, OUT_F64, P><<<nb, 32 * kEpiWarps, 0, st>>>(a); break;
-        case OUT_PART: epilogue_kernel<TDENSE, MODE, OUT_PART, P><<<nb, 32 * kEpiWarps, 0, st>>>(a); break;
-        default: epilogue_kernel<TDENSE, MODE, OUT_EULER, P><<<nb, 32 * kEpiWarps, 0, st>>>(a); break;
+        case OUT_F32: epilogue_kernel<TDENSE, MODE, OUT_F32, P, W><<<nb, 32 * W, 0, st>>>(a); break;
+        case OUT_F64: epilogue_kernel<TDENSE, MODE, OUT_F64, P, W><<<nb, 32 * W, 0, st>>>(a); break;
+        case OUT_PART: epilogue_kernel<TDENSE, MODE, OUT_PART, P, W><<<nb, 32 * W, 0, st>>>(a); break;
+        default: epilogue_kernel<TDENSE, MODE, OUT_EULER, P, W><<<nb, 32 * W, 0, st>>>(a); break;
     }
+}
+
+template <int TDENSE, int MODE>
+static void epi_launch_shape(int out, cudaStream_t st, const EpiArgs &a) {
+    // two particles per lane needs an even first row (aligned loads) and no shard shares
+    if (a.n <= SD_EPI_SMALL_N)
+        epi_launch<TDENSE, MODE, 1, 2 * kEpiWarps>(out, st, a);
+    else if (MODE == MODE_FP32C && kEpiPairs && (a.row0 & 1) == 0 && !a.sh.pall)
+        epi_launch<TDENSE, MODE, MODE == MODE_FP32C ? 2 : 1, kEpiWarps>(out, st, a);
+    else
+        epi_launch<TDENSE, MODE, 1, kEpiWarps>(out, st, a);
 }
 
 template <int TDENSE>
 static void epi_launch_mode(int mode, int out, cudaStream_t st, const EpiArgs &a) {
     switch (mode) {
-        case MODE_FP32C:
-            // two particles per lane needs an even first row (aligned loads) and no shard shares
-            if (kEpiPairs && (a.row0 & 1) == 0 && !a.sh.pall)
-                epi_launch<TDENSE, MODE_FP32C, 2>(out, st, a);
-            else
-                epi_launch<TDENSE, MODE_FP32C, 1>(out, st, a);
-            break;
-        case MODE_FP64: epi_launch<TDENSE, MODE_FP64, 1>(out, st, a); break;
-        default: epi_launch<TDENSE, MODE_FP32, 1>(out, st, a); break;
+        case MODE_FP32C: epi_launch_shape<TDENSE, MODE_FP32C>(out, st, a); break;
+        case MODE_FP64: epi_launch_shape<TDENSE, MODE_FP64>(out, st, a); break;
+        default: epi_launch_shape<TDENSE, MODE_FP32>(out, st, a); break;
     }
 }
 

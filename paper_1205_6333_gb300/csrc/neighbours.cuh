@@ -51,9 +51,141 @@ __device__ __forceinline__ void for_each_neighbour_part(const CellList &c, int i
     }
 }
 
-// Nearest-image FP64 separation r_i - r_j (identity in unbounded dimensions).
+// ---------------------------------------------------------------- mirrors and bins
+
+// Entry i of a mirror: (x, y, z, 0) in the AoS array and, if present, the SoA copy.
+template <typename V4>
+__device__ __forceinline__ void put_mirror(V4 *aos, float *soa, int npad, int i, double x, double y, double z) {
+    V4 v;
+    v.x = x;
+    v.y = y;
+    v.z = z;
+    v.w = 0;
+    aos[i] = v;
+    if (soa) {
+        soa[i] = static_cast<float>(x);
+        soa[npad + i] = static_cast<float>(y);
+        soa[2 * static_cast<size_t>(npad) + i] = static_cast<float>(z);
+    }
+}
+
+// u wrapped into [0, L) in a periodic dimension (L > 0), unchanged otherwise.
+__device__ __forceinline__ double wrap_box(double u, double L, double invL) {
+    return L > 0.0 ? u - L * floor(u * invL) : u;
+}
+
+// Mirror entry of a position: relative to particle 0 (only differences enter the
+// pair terms, and small coordinates keep FP32 separations accurate), wrapped into
+// the box in periodic dimensions (the pair terms take the nearest image).
+template <typename V4>
+__device__ __forceinline__ void put_pos_mirror(V4 *m, float *soa, int npad, int i, const double *x, const Box &b) {
+    const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
+    put_mirror(m, soa, npad, i, wrap_box(px - x[0], b.L[0], b.invL[0]), wrap_box(py - x[1], b.L[1], b.invL[1]),
+               wrap_box(pz - x[2], b.L[2], b.invL[2]));
+}
+
+__device__ __forceinline__ int cell_coord(double x, double inv_h) {
+    double c = floor(x * inv_h);
+    c = fmin(fmax(c, -1.0e9), 1.0e9);  // keep the integer in range for absurd coordinates
+    return static_cast<int>(c);
+}
+
+// Cell coordinate in dimension d: nc[d] cells over [0, L) of the wrapped coordinate
+// in a periodic dimension, cells of side h otherwise.
+__device__ __forceinline__ int cell_coord_d(const CellList &c, int d, double x) {
+    const int nc = c.nc[d];
+    if (nc <= 0) return cell_coord(x, c.inv_h);
+    const int k = static_cast<int>(floor(wrap_box(x, c.box.L[d], c.box.invL[d]) * c.box.invL[d] * nc));
+    return k < 0 ? 0 : (k >= nc ? nc - 1 : k);
+}
+
+// Particle i's cell and bucket; counts it there.
+__device__ __forceinline__ void bin_particle(const CellList &c, int i, double px, double py, double pz) {
+    const int cx = cell_coord_d(c, 0, px);
+    const int cy = cell_coord_d(c, 1, py);
+    const int cz = cell_coord_d(c, 2, pz);
+    c.cell[i] = make_int4(cx, cy, cz, 0);
+    const uint32_t k = cell_hash(cx, cy, cz, c.H);
+    c.key[i] = k;
+    atomicAdd(&c.cnt[k], 1);
+}
+
+constexpr int kScanPer = 16;   // buckets a thread scans
+
+// Exclusive scan of kScanPer values per thread across a block; returns the
+// block total.  Warp shuffles within warps, shared memory across warps.
+template <int NT>
+__device__ __forceinline__ int block_exclusive_scan(int v[kScanPer], int *s_warp) {
+    int tsum = 0;
+    for (int k = 0; k < kScanPer; ++k) {
+        const int t = v[k];
+        v[k] = tsum;
+        tsum += t;
+    }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int incl = tsum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    if (wid == 0) {
+        int w = (lane < NT / 32) ? s_warp[lane] : 0;
+        int wi = w;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += y;
+        }
+        s_warp[lane] = wi - w;  // exclusive warp offsets
+        if (lane == 31) s_warp[32] = wi;
+    }
+    __syncthreads();
+    const int off = s_warp[wid] + incl - tsum;
+    for (int k = 0; k < kScanPer; ++k) v[k] += off;
+    const int total = s_warp[32];
+    __syncthreads();
+    return total;
+}
+
+// Particle i takes a place in its bucket by counting the bucket's occupancy down, which
+// leaves every counter at zero for the next build (no memset).
+__device__ __forceinline__ void scatter_particle(const uint32_t *key, const int *start, int *cnt, int *sorted, int i,
+                                                 int *err) {
+    const uint32_t k = key[i];
+    const int pos = start[k] + atomicSub(&cnt[k], 1) - 1;
+    if (pos >= start[k] && pos < start[k + 1])   // always, unless a counter was left non-zero
+        sorted[pos] = i;
+    else
+        atomicOr(err, DEV_ERR_BOUNDS);
+}
+
+// Sort bucket b by particle index (buckets hold ~1 particle; a bucket larger
+// than 256 -- only possible for unphysically dense input -- stays unsorted, which
+// changes only the FP64 summation order of its near pairs).
+__device__ __forceinline__ void sort_bucket(const int *start, int *sorted, int b) {
+    const int s0 = start[b], s1 = start[b + 1];
+    if (s1 - s0 < 2 || s1 - s0 > 256) return;
+    for (int p = s0 + 1; p < s1; ++p) {
+        const int v = sorted[p];
+        int q = p - 1;
+        while (q >= s0 && sorted[q] > v) {
+            sorted[q + 1] = sorted[q];
+            --q;
+        }
+        sorted[q + 1] = v;
+    }
+}
+
+// Nearest-image FP64 separation r_i - r_j (identity in unbounded dimensions).  Most pairs
+// need no image: |d| below half a period rounds to zero periods, and a comparison of the upper
+// words (integers) says so without the twelve FP64 operations (two a clock and SM).
+__device__ __forceinline__ bool within_half(double d, double L) {
+    return L == 0.0 || (__double2hiint(d) & 0x7fffffff) < __double2hiint(0.5 * L);
+}
 __device__ __forceinline__ void box_image(const Box &b, double &dx, double &dy, double &dz) {
     if (!b.periodic) return;
+    if (within_half(dx, b.L[0]) && within_half(dy, b.L[1]) && within_half(dz, b.L[2])) return;
     dx = min_image_f64(dx, b.L[0], b.invL[0]);
     dy = min_image_f64(dy, b.L[1], b.invL[1]);
     dz = min_image_f64(dz, b.L[2], b.invL[2]);

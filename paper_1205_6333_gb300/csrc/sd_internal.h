@@ -153,12 +153,11 @@ struct CellList {
     Box box;
     int nc[3] = {0, 0, 0};          // cells per periodic dimension (0: unbounded)
     int H = 0;
-    int nblk = 0;          // scan blocks
     int4 *cell = nullptr;  // [n] integer cell coordinates (w unused)
     uint32_t *key = nullptr;  // [n] bucket of each particle
     int *cnt = nullptr;    // [H] occupancy (zero between builds)
     int *start = nullptr;  // [H+1]
-    int *bsum = nullptr;   // [nblk]
+    int *bsum = nullptr;   // [scan chunks]
     int *sorted = nullptr; // [n]
     int n = 0;             // particles binned
     int *err = nullptr;    // device error word (debug index checks)
@@ -178,6 +177,25 @@ struct Mirror {
     void *aos = nullptr;
     float *soa = nullptr;
 };
+
+// Dynamic shared memory of a launch of `grid` CTAs, `occ` of which fit an SM with `need`
+// bytes: where the grid does not fill them, as much as keeps an SM from taking more than an
+// even share.  (CTAs go where there is room, and beside a kernel on another stream that is
+// here and there at first: an FP64 step of 1,500 particles, 78 CTAs, took 1.25 ms instead of 0.21.)
+inline size_t spread_smem(int num_sms, int grid, int occ, size_t need, size_t limit) {
+    const size_t per = static_cast<size_t>((grid + num_sms - 1) / num_sms);
+    if (per >= static_cast<size_t>(occ)) return need;
+    const size_t s = ((228 * 1024 / (per + 1) - 1024) / 128 + 1) * 128;   // (an SM's 228 KB; 1 KB a CTA is the system's)
+    return s < need ? need : (s < limit ? s : limit);
+}
+// The most dynamic shared memory a launch of fn can have, and the attribute that allows it.
+inline cudaError_t allow_smem(const void *fn, size_t &limit) {
+    cudaFuncAttributes at{};
+    cudaError_t e = cudaFuncGetAttributes(&at, fn);
+    if (e != cudaSuccess) return e;
+    limit = 227 * 1024 - ((at.sharedSizeBytes + 127) & ~static_cast<size_t>(127));
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(limit));
+}
 
 struct Profiler {
     bool on = false;
@@ -222,6 +240,7 @@ struct sd_handle {
     int cur = 0;
     bool pos_set = false;
     bool cells_valid = false;             // cell list matches x64[cur]
+    bool near_valid = false;              // ... and near_ent holds its candidate pairs (meaningful while cells_valid)
 
     double *fext64 = nullptr;   // [n*3] per-particle external forces
     double *F64 = nullptr;      // [n*3] total force of the current step
@@ -242,6 +261,7 @@ struct sd_handle {
     unsigned *small_sync = nullptr;  // [3] words and
     ulonglong2 *small_xch = nullptr; // [2][3 n] the position exchange of the small path (small.cu)
     int dense_occ = 0, vjp_occ = 0;
+    size_t dense_limit = 0, vjp_limit = 0;   // most dynamic shared memory of their kernels (allow_smem)
     int sym_nt = 128;   // threads per CTA of the symmetric kernel's chosen block shape
 
     sd::CellList cl;
@@ -319,14 +339,13 @@ void prof_end(sd_handle *h, int kind, cudaStream_t st);
 // cells.cu
 cudaError_t launch_stage_pos(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm);
 cudaError_t launch_stage_forces(sd_handle *h, cudaStream_t st, const void *src, int src_dtype, int add_ext,
-                                double *dst64, Mirror dstm);
-// xref != nullptr: a Verlet-list build (copies x64 to xref and clears the rebuild
-// request); otherwise any build requests a rebuild of the step's list.
+                                double *dst64, Mirror dstm, const void *src2 = nullptr, double *dst2 = nullptr,
+                                Mirror dstm2 = Mirror{});
+// xref != nullptr: a Verlet list's build (copies x64 to xref; the mirror is the check's).
 cudaError_t launch_build_cells(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm,
                                double *xref = nullptr);
-// Verlet step: the mirror of x64, the clamp flag reset, and the rebuild decision
-// (displacements relative to particle 0 since xref; list overflow) in d_vl[0].
-cudaError_t launch_verlet_check(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm);
+// The same in a Verlet step, if its check asked for it.
+cudaError_t launch_rebuild_cells(sd_handle *h, cudaStream_t st, const double *x64);
 cudaError_t launch_forces_rep(sd_handle *h, cudaStream_t st, const double *x64);
 // Verlet step with soft repulsion: the forces from the steps' near-pair list.
 cudaError_t launch_forces_list(sd_handle *h, cudaStream_t st, const double *x64);
@@ -340,11 +359,16 @@ cudaError_t launch_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm
 // the pass needs no memset of its own.
 cudaError_t launch_near(sd_handle *h, cudaStream_t st, const double *x64, const void *posm, const double *F64,
                         const void *frcm, bool count_zeroed = false);
-// The two halves of the near pass: the candidate list (cutoff r_near, or r_near + skin
-// for a Verlet list, which is then sorted by partner within each particle) and the
-// FP64 terms of the listed pairs.
+// Verlet step: the mirror of x64, the clamp flag and the rebuild request; then the list, if it
+// was asked for (build: unconditionally).
+cudaError_t launch_verlet_check(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm);
+cudaError_t launch_verlet_rebuild(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, bool build = false);
+// The cell list, the mirror and the candidate list of the near pass (cutoff r_near).
+cudaError_t launch_near_lists(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm, const double *F64,
+                              const void *frcm);
+// The candidate list alone (the cell list is there); the FP64 terms of the listed pairs.
 cudaError_t launch_near_collect(sd_handle *h, cudaStream_t st, const double *x64, const void *posm,
-                                const double *F64, const void *frcm, bool count_zeroed, bool verlet_list);
+                                const double *F64, const void *frcm, bool count_zeroed);
 cudaError_t launch_near_pairs(sd_handle *h, cudaStream_t st, const double *x64, const void *posm, const double *F64,
                               const void *frcm, bool verlet_step = false);
 cudaError_t launch_epilogue(sd_handle *h, cudaStream_t st, int out, const double *x64, const void *posm,
