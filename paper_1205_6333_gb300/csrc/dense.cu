@@ -56,7 +56,7 @@ __device__ __forceinline__ void dense_pair(typename DenseT<MODE>::S xi, typename
                                            typename DenseT<MODE>::S &ax, typename DenseT<MODE>::S &ay,
                                            typename DenseT<MODE>::S &az) {
     if constexpr (MODE == MODE_FP64)
-        pair_f64<TENSOR, PER>(xi, yi, zi, p, f, c, ax, ay, az);
+        pair_dir_f64<TENSOR, PER>(xi, yi, zi, p, f, c, ax, ay, az);   // (divided by c1)
     else
         pair_f32<TENSOR, true, PER>(xi, yi, zi, p, f, c, ax, ay, az);
 }
@@ -122,9 +122,10 @@ __global__ void __launch_bounds__(kNT) dense_kernel(const typename DenseT<MODE>:
                 vy = static_cast<double>(hy[k]) + static_cast<double>(ly[k]);
                 vz = static_cast<double>(hz[k]) + static_cast<double>(lz[k]);
             } else {
-                vx = static_cast<double>(ax[k]);
-                vy = static_cast<double>(ay[k]);
-                vz = static_cast<double>(az[k]);
+                const double m = MODE == MODE_FP64 ? c.c1_d : 1.0;
+                vx = m * static_cast<double>(ax[k]);
+                vy = m * static_cast<double>(ay[k]);
+                vz = m * static_cast<double>(az[k]);
             }
             dst[i] = vx;
             dst[npad + i] = vy;
@@ -622,7 +623,9 @@ __global__ void __launch_bounds__(NT, SD_SYM_MINB) dense_sym_kernel(const float 
 // counterpart of dense_sym_kernel.  GB300 issues FP64 at a small fraction of its
 // FP32 rate, so this kernel is bound by the FP64 pipe alone and its only aim is
 // fewer FP64 operations per pair: r, 1/r, A and B are formed once per unordered
-// pair (pair_sym_f64), 19 FP64 operations per ordered pair against 30 directed.
+// pair (pair_sym_f64), 35 FP64 operations against 2 x 25 directed.  With the clamp, the
+// root's conversions and c1 on the FP64 pipe too (40 and
+// more) the product at N = 8,192 took 2,533 us; now 2,245.
 //   * blocks of kB64 = 128 particles, one target per thread (128 threads); a tile
 //     is an unordered block pair (ib <= jb), partitioned over the persistent grid
 //     as in dense_sym_kernel; the positions and forces of block jb (dbl4, AoS) are
@@ -702,9 +705,9 @@ __global__ void __launch_bounds__(kB64) dense_sym64_kernel(const dbl4 *__restric
     auto flush = [&](int ib) {
         const int slot = cta - geom_first(g, ib);
         double *dst = part + static_cast<size_t>(slot) * 3 * npad + static_cast<size_t>(ib) * B + tid;
-        dst[0] = ax;
-        dst[npad] = ay;
-        dst[2 * static_cast<size_t>(npad)] = az;
+        dst[0] = c.c1_d * ax;
+        dst[npad] = c.c1_d * ay;
+        dst[2 * static_cast<size_t>(npad)] = c.c1_d * az;
     };
 
     int ib = ib0, jb = jb0;
@@ -732,7 +735,7 @@ __global__ void __launch_bounds__(kB64) dense_sym64_kernel(const dbl4 *__restric
         const bool diag = ib == jb;
         if (diag) {
 #pragma unroll 2
-            for (int jj = 0; jj < B; ++jj) pair_f64<TENSOR, PER>(xi, yi, zi, P[jj], Fq[jj], c, ax, ay, az);
+            for (int jj = 0; jj < B; ++jj) pair_dir_f64<TENSOR, PER>(xi, yi, zi, P[jj], Fq[jj], c, ax, ay, az);
         } else {
             const int nxt = (lane + 1) & 31;
 #pragma unroll 1
@@ -759,7 +762,7 @@ __global__ void __launch_bounds__(kB64) dense_sym64_kernel(const dbl4 *__restric
                 double v = s_jacc[e];
 #pragma unroll
                 for (int w = 1; w < NW; ++w) v += s_jacc[w * 3 * B + e];
-                dst[e] = v;
+                dst[e] = c.c1_d * v;
             }
             __syncthreads();  // s_jacc free for the next tile
         }

@@ -268,6 +268,8 @@ __device__ __forceinline__ void pair_sym_f32x2(f2 XI, f2 YI, f2 ZI, f2 GX, f2 GY
 
 // ---------------------------------------------------------------- dense FP64
 
+// What the FP64 all-pairs kernels add for a pair, to rounding (the near pass and the epilogue
+// take it out of the sums).
 template <int TENSOR, bool PER = false>
 __device__ __forceinline__ void pair_f64(double xi, double yi, double zi, dbl4 p, dbl4 f, const PairConst &c,
                                          double &ax, double &ay, double &az) {
@@ -299,46 +301,6 @@ __device__ __forceinline__ void pair_f64(double xi, double yi, double zi, dbl4 p
     az = __fma_rn(s, dz, __fma_rn(A, f.z, az));
 }
 
-// The pair (i, j) used in both directions in FP64 (mu_ij = mu_ji, Sec. 2.2): r, r^2,
-// 1/r, A and B once, then
-//   a += mu(r_i - r_j) F_j / mu0    (target i),   b += mu(r_j - r_i) F_i / mu0   (source j).
-// r_j - r_i = -(r_i - r_j) exactly and every step is a round-to-nearest operation,
-// so each direction is bit-identical to pair_f64 evaluated for that ordered pair.
-template <int TENSOR, bool PER = false>
-__device__ __forceinline__ void pair_sym_f64(double xi, double yi, double zi, double gx, double gy, double gz,
-                                             const dbl4 &p, const dbl4 &f, const PairConst &c, double &ax,
-                                             double &ay, double &az, double &bx, double &by, double &bz) {
-    double dx = __dsub_rn(xi, p.x);
-    double dy = __dsub_rn(yi, p.y);
-    double dz = __dsub_rn(zi, p.z);
-    if (PER) {
-        dx = min_image_f64(dx, c.Ld[0], c.invLd[0]);
-        dy = min_image_f64(dy, c.Ld[1], c.invLd[1]);
-        dz = min_image_f64(dz, c.Ld[2], c.invLd[2]);
-    }
-    double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-    r2 = fmax(r2, c.r2min_d);
-    const double ri = rsqrt_nr64(r2);
-    const double ri2 = __dmul_rn(ri, ri);
-    double A, B;
-    if (TENSOR == T_OSEEN) {
-        A = __dmul_rn(c.c1_d, ri);
-        B = __dmul_rn(A, ri2);
-    } else {
-        A = __dmul_rn(ri, __fma_rn(c.c3_d, ri2, c.c1_d));
-        const double ri3 = __dmul_rn(ri, ri2);
-        B = __dmul_rn(ri3, __fma_rn(c.m3c3_d, ri2, c.c1_d));
-    }
-    const double s = __dmul_rn(B, __fma_rn(dz, f.z, __fma_rn(dy, f.y, __dmul_rn(dx, f.x))));
-    ax = __fma_rn(s, dx, __fma_rn(A, f.x, ax));
-    ay = __fma_rn(s, dy, __fma_rn(A, f.y, ay));
-    az = __fma_rn(s, dz, __fma_rn(A, f.z, az));
-    const double u = __dmul_rn(B, __fma_rn(dz, gz, __fma_rn(dy, gy, __dmul_rn(dx, gx))));
-    bx = __fma_rn(u, dx, __fma_rn(A, gx, bx));
-    by = __fma_rn(u, dy, __fma_rn(A, gy, by));
-    bz = __fma_rn(u, dz, __fma_rn(A, gz, bz));
-}
-
 // A / c1 and B / c1 of the Rotne-Prager / Oseen form in FP64 (the sums are multiplied by c1
 // once per particle): 1/r + k/r^3 and 1/r^3 - 3k/r^5 with k = c3 / c1, nine FP64 operations
 // with the root (Oseen: six) and no conversions.
@@ -356,6 +318,52 @@ __device__ __forceinline__ void profile64(double r2, const PairConst &c, double 
 
 // x < y for non-negative FP64 values, in integer operations.
 __device__ __forceinline__ bool less_pos64(double x, double y) { return __double_as_longlong(x) < __double_as_longlong(y); }
+
+// r, A / c1 and B / c1 of a pair of the FP64 all-pairs kernels, with r^2 clamped to (2a)^2 (an
+// integer comparison: FP64 issues two operations a clock and SM, integers 64 and more).
+template <int TENSOR, bool PER>
+__device__ __forceinline__ void pair_head64(double xi, double yi, double zi, const dbl4 &p, const PairConst &c,
+                                            double (&d)[3], double &A, double &B) {
+    d[0] = __dsub_rn(xi, p.x);
+    d[1] = __dsub_rn(yi, p.y);
+    d[2] = __dsub_rn(zi, p.z);
+    if (PER)
+        for (int k = 0; k < 3; ++k) d[k] = min_image_f64(d[k], c.Ld[k], c.invLd[k]);
+    double r2 = __fma_rn(d[2], d[2], __fma_rn(d[1], d[1], __dmul_rn(d[0], d[0])));
+    r2 = less_pos64(r2, c.r2min_d) ? c.r2min_d : r2;
+    profile64<TENSOR>(r2, c, A, B);
+}
+__device__ __forceinline__ void pair_add64(const double (&d)[3], double A, double B, double fx, double fy, double fz,
+                                           double &ax, double &ay, double &az) {
+    const double s = __dmul_rn(B, __fma_rn(d[2], fz, __fma_rn(d[1], fy, __dmul_rn(d[0], fx))));
+    ax = __fma_rn(s, d[0], __fma_rn(A, fx, ax));
+    ay = __fma_rn(s, d[1], __fma_rn(A, fy, ay));
+    az = __fma_rn(s, d[2], __fma_rn(A, fz, az));
+}
+
+// One pair of the directed FP64 sum, divided by c1 (the kernel multiplies its sums): 25 FP64
+// operations (RP).
+template <int TENSOR, bool PER = false>
+__device__ __forceinline__ void pair_dir_f64(double xi, double yi, double zi, const dbl4 &p, const dbl4 &f,
+                                             const PairConst &c, double &ax, double &ay, double &az) {
+    double d[3], A, B;
+    pair_head64<TENSOR, PER>(xi, yi, zi, p, c, d, A, B);
+    pair_add64(d, A, B, f.x, f.y, f.z, ax, ay, az);
+}
+
+// The pair (i, j) used in both directions in FP64 (mu_ij = mu_ji, Sec. 2.2): r, r^2,
+// 1/r, A and B once, then
+//   a += mu(r_i - r_j) F_j / (mu0 c1)    (target i),   b += mu(r_j - r_i) F_i / (mu0 c1)   (source j):
+// 35 FP64 operations (RP).
+template <int TENSOR, bool PER = false>
+__device__ __forceinline__ void pair_sym_f64(double xi, double yi, double zi, double gx, double gy, double gz,
+                                             const dbl4 &p, const dbl4 &f, const PairConst &c, double &ax,
+                                             double &ay, double &az, double &bx, double &by, double &bz) {
+    double d[3], A, B;
+    pair_head64<TENSOR, PER>(xi, yi, zi, p, c, d, A, B);
+    pair_add64(d, A, B, f.x, f.y, f.z, ax, ay, az);
+    pair_add64(d, A, B, gx, gy, gz, bx, by, bz);
+}
 
 // ---------------------------------------------------------------- exact FP64 profile
 
