@@ -299,6 +299,9 @@ static sd_status run_steps(sd_handle *h, double dt, int64_t nsteps) {
 // The adjoint's work on one checkpoint segment of K steps, on stream st:
 //   recompute (part 0): x_{k+1} = x_k + dt v(x_k) into seg, k = 0 .. K-2;
 //   reverse (part 1), k = K-1 .. 0: W = lambda; lambda += dt (dv/dx(x_k))^T W; gF += dt mu(x_k) W.
+// A reverse step has a Verlet step's shape: the check kernel, the all-pairs kernel with the
+// rebuild and the listed pairs' FP64 terms beside it, and the epilogue, which leaves lambda's
+// mirror for the next one.
 static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int64_t len, int part) {
     const size_t n3 = 3 * static_cast<size_t>(h->n);
     auto segx = [&](int64_t k) { return h->seg + static_cast<size_t>(k) * n3; };
@@ -313,12 +316,21 @@ static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int
         return e;
     }
     for (int64_t k = len - 1; k >= 0 && e == cudaSuccess; --k) {
-        e = launch_stage_forces(h, st, h->lam, SD_DTYPE_F64, 0, h->Wa64, h->wam);
-        if (e == cudaSuccess) e = launch_build_cells(h, st, segx(k), h->posm);
+        const VjpInput in{segx(k), h->F64, h->frcm, h->lam, h->verlet};
+        cudaStream_t side = h->verlet ? h->side : st;
+        if (h->verlet) {
+            e = launch_verlet_check(h, st, segx(k), h->posm);
+            if (e == cudaSuccess) e = cudaEventRecord(h->ev_fork, st);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(side, h->ev_fork, 0);
+            if (e == cudaSuccess) e = launch_verlet_rebuild(h, side, segx(k), h->posm);
+        } else {
+            e = launch_near_lists(h, st, segx(k), h->posm, h->F64, h->frcm.aos);
+        }
+        if (e == cudaSuccess) e = launch_vjp_near(h, side, in);
+        if (h->verlet && e == cudaSuccess) e = cudaEventRecord(h->ev_join, side);
         if (e == cudaSuccess) e = launch_vjp_dense(h, st, h->posm, h->frcm, h->wam, h->part, h->part2);
-        if (e == cudaSuccess)
-            e = launch_vjp_epilogue(h, st, segx(k), h->posm.aos, h->F64, h->frcm.aos, h->Wa64, h->wam.aos, -1,
-                                    nullptr, nullptr, dt, h->lam, h->gFacc);
+        if (h->verlet && e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
+        if (e == cudaSuccess) e = launch_vjp_epilogue(h, st, in, -1, nullptr, nullptr, dt, h->lam, h->gFacc);
     }
     return e;
 }
@@ -553,11 +565,13 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
         if (h->small.on && (!dalloc_t(h, h->small_sync, 3) || !dalloc_t(h, h->small_xch, 2 * n3)))
             return fail(SD_ERR_OOM, "device allocation of the small systems' exchange");
         if (!h->part || !h->part2) return fail(SD_ERR_OOM, "device allocation of partial sums");
-        if (h->geom.sym) {
+        {   // one buffer: the product's and the VJP's source-side sums are not live together
             const size_t es = h->mode == MODE_FP64 ? sizeof(double) : sizeof(float);
-            h->jpart_bytes = static_cast<size_t>(h->geom.nT) * 3 * h->geom.I * es;
-            h->jpart = dalloc(h, h->jpart_bytes);
-            if (!h->jpart) return fail(SD_ERR_OOM, "device allocation of source-side partial sums");
+            const size_t nd = h->geom.sym ? static_cast<size_t>(h->geom.nT) * 3 * h->geom.I : 0;
+            const size_t nv = h->geomv.sym ? static_cast<size_t>(h->geomv.nT) * 6 * h->geomv.I : 0;
+            h->jpart_bytes = std::max(nd, nv) * es;
+            if (h->jpart_bytes) h->jpart = dalloc(h, h->jpart_bytes);
+            if (h->jpart_bytes && !h->jpart) return fail(SD_ERR_OOM, "device allocation of source-side partial sums");
         }
     }
 
@@ -1035,16 +1049,15 @@ sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, 
         gXd = gX ? b + 2 * bytes : nullptr;
         gFd = gF ? b + 3 * bytes : nullptr;
     }
-    sd_status s = launch_check(launch_stage_forces(h, h->stream, Fd, dtype, 0, h->Fa64, h->frcam), "stage F");
-    if (s == SD_OK) s = launch_check(launch_stage_forces(h, h->stream, Wd, dtype, 0, h->Wa64, h->wam), "stage W");
-    if (s == SD_OK) s = ensure_cells(h);
+    sd_status s = launch_check(launch_stage_forces(h, h->stream, Fd, dtype, 0, h->Fa64, h->frcam, Wd, h->Wa64, h->wam),
+                               "stage F and W");
+    if (s == SD_OK) s = launch_check(near_list(h, true), "near pass");
+    const VjpInput vin{h->x64[h->cur], h->Fa64, h->frcam, h->Wa64, false};
+    if (s == SD_OK) s = launch_check(launch_vjp_near(h, h->stream, vin), "near pass");
     if (s == SD_OK)
-        s = launch_check(launch_vjp_dense(h, h->stream, h->posm, h->frcam, h->wam, h->part, h->part2),
-                         "vjp kernel");
+        s = launch_check(launch_vjp_dense(h, h->stream, h->posm, h->frcam, h->wam, h->part, h->part2), "vjp kernel");
     if (s == SD_OK)
-        s = launch_check(launch_vjp_epilogue(h, h->stream, h->x64[h->cur], h->posm.aos, h->Fa64, h->frcam.aos,
-                                             h->Wa64, h->wam.aos, dtype, gXd, gFd, 0.0, nullptr, nullptr),
-                         "vjp epilogue");
+        s = launch_check(launch_vjp_epilogue(h, h->stream, vin, dtype, gXd, gFd, 0.0, nullptr, nullptr), "vjp epilogue");
     if (s != SD_OK) return s;
     if (!on_device) {
         if (gX) SD_CUDA(cudaMemcpyAsync(gX, gXd, bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1096,7 +1109,12 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
     // forward with checkpoints, segment by segment through the step graphs (the state
     // ping-pongs through x64[0], x64[1])
     SD_CUDA(cudaMemcpyAsync(h->ckpt, h->x64[c0], xb, cudaMemcpyDeviceToDevice, st));
-    for (int64_t sg = 0; sg < nseg; ++sg) {
+    // (the last segment's steps are those that its recompute takes: x_T itself is not needed)
+    if (h->verlet && !h->list_set) {
+        sd_status ss = build_list(h);
+        if (ss != SD_OK) return ss;
+    }
+    for (int64_t sg = 0; sg + 1 < nseg; ++sg) {
         const int64_t len = std::min(K, nsteps - sg * K);
         sd_status ss = run_steps(h, dt, len);
         if (ss != SD_OK) return ss;
@@ -1111,6 +1129,10 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
     else
         SD_CUDA(cudaMemcpyAsync(h->lam, gxT, xb, cudaMemcpyHostToDevice, st));
     SD_CUDA(cudaMemsetAsync(h->gFacc, 0, xb, st));
+    {
+        sd_status ss = launch_check(launch_stage_forces(h, st, h->lam, SD_DTYPE_F64, 0, h->Wa64, h->wam), "stage lambda");
+        if (ss != SD_OK) return ss;
+    }
     // reverse sweep, last segment first: recompute the segment's positions from its
     // checkpoint, then walk it backwards.  Full segments replay cached graphs (eager
     // with the profiler on, and for a shorter last segment).

@@ -521,50 +521,108 @@ __device__ __forceinline__ void vjp_pair_f32x2(f2 XI, f2 YI, f2 ZI, f2 FIx, f2 F
     M[2] = fma2(bWj, dz, fma2(A, WZ, M[2]));
 }
 
-// The same pair in FP64 with the clamp (what the FP64 dense VJP kernel adds).
-template <int TENSOR, bool PER = false>
-__device__ __forceinline__ void vjp_pair_f64(double xi, double yi, double zi, double3 Fi, double3 Wi, dbl4 p,
-                                             dbl4 f, dbl4 w, const PairConst &c, double3 &m, double3 &g) {
-    double dx = __dsub_rn(xi, p.x);
-    double dy = __dsub_rn(yi, p.y);
-    double dz = __dsub_rn(zi, p.z);
+// The pairs (i, j0), (i, j1) used in both directions, operands as in vjp_pair_f32x2: from one
+// r, 1/r and profile
+//   M += A Wj + B (r.Wj) r,   JM += A Wi + B (r.Wi) r   (rows i and j of mu W),
+//   G += g,                   JG += g                   (the pair's gradient with respect to x_j is -g).
+// FIRST: JM and JG are set, not added to; a caller with several targets adds their terms
+// before they join the long sums (fewer roundings at the sums' size).
+// 76 packed operations for four ordered pairs, against 64 for two in vjp_pair_f32x2.
+template <int TENSOR, bool PER, bool FIRST>
+__device__ __forceinline__ void vjp_sym_f32x2(f2 XI, f2 YI, f2 ZI, const f2 (&FI)[3], const f2 (&WI)[3], f2 PX, f2 PY,
+                                              f2 PZ, f2 FX, f2 FY, f2 FZ, f2 WX, f2 WY, f2 WZ, const VjpConst2 &c,
+                                              f2 (&M)[3], f2 (&G)[3], f2 (&JM)[3], f2 (&JG)[3]) {
+    f2 dx = sub2(XI, PX);
+    f2 dy = sub2(YI, PY);
+    f2 dz = sub2(ZI, PZ);
     if (PER) {
-        dx = min_image_f64(dx, c.Ld[0], c.invLd[0]);
-        dy = min_image_f64(dy, c.Ld[1], c.invLd[1]);
-        dz = min_image_f64(dz, c.Ld[2], c.invLd[2]);
+        dx = min_image2(dx, c.negL[0], c.invL[0]);
+        dy = min_image2(dy, c.negL[1], c.invL[1]);
+        dz = min_image2(dz, c.negL[2], c.invL[2]);
     }
-    double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-    r2 = fmax(r2, c.r2min_d);
-    const double ri = rsqrt_nr64(r2);
-    const double ri2 = ri * ri;
-    const double ri3 = ri * ri2;
-    const double ri5 = ri3 * ri2;
+    float ra, rb;
+    upk2(fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), ra, rb);
+    const f2 ri = pk2(rsqrt_sfu(fmaxf(ra, c.r2min)), rsqrt_sfu(fmaxf(rb, c.r2min)));
+    const f2 ri2 = mul2(ri, ri), ri3 = mul2(ri, ri2), ri5 = mul2(ri3, ri2);
+    f2 A, Bv, dA, dB;
+    if (TENSOR == T_OSEEN) {
+        A = mul2(c.c1, ri);
+        Bv = mul2(c.c1, ri3);
+        dA = mul2(c.nc1, ri3);
+        dB = mul2(c.n3c1, ri5);
+    } else {
+        A = mul2(ri, fma2(c.c3, ri2, c.c1));
+        Bv = mul2(ri3, fma2(c.m3c3, ri2, c.c1));
+        dA = mul2(ri3, fma2(c.m3c3, ri2, c.nc1));
+        dB = mul2(ri5, fma2(c.n5m3c3, ri2, c.n3c1));
+    }
+    const f2 Wir = fma2(dz, WI[2], fma2(dy, WI[1], mul2(dx, WI[0])));
+    const f2 Fir = fma2(dz, FI[2], fma2(dy, FI[1], mul2(dx, FI[0])));
+    const f2 Wjr = fma2(dz, WZ, fma2(dy, WY, mul2(dx, WX)));
+    const f2 Fjr = fma2(dz, FZ, fma2(dy, FY, mul2(dx, FX)));
+    const f2 U = fma2(WZ, FI[2], fma2(WY, FI[1], fma2(WX, FI[0], fma2(WI[2], FZ, fma2(WI[1], FY, mul2(WI[0], FX))))));
+    const f2 cr = fma2(dB, fma2(Wjr, Fir, mul2(Wir, Fjr)), mul2(dA, U));
+    const f2 bFj = mul2(Bv, Fjr), bWi = mul2(Bv, Wir), bFi = mul2(Bv, Fir), bWj = mul2(Bv, Wjr);
+    const f2 d[3] = {dx, dy, dz}, F[3] = {FX, FY, FZ}, W[3] = {WX, WY, WZ};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const f2 g = fma2(cr, d[k], fma2(WI[k], bFj, fma2(F[k], bWi, fma2(W[k], bFi, mul2(FI[k], bWj)))));
+        G[k] = add2(G[k], g);
+        JG[k] = FIRST ? g : add2(JG[k], g);
+        M[k] = fma2(bWj, d[k], fma2(A, W[k], M[k]));
+        JM[k] = fma2(bWi, d[k], FIRST ? mul2(A, WI[k]) : fma2(A, WI[k], JM[k]));
+    }
+}
+
+// The FP64 pair (i, j) in both directions, divided by c1 (the epilogue multiplies the sums):
+// t = x, F, W of the target, s = those of the source.  77 FP64 operations (RP) with the
+// clamp and the root's seed in integer operations, against 2 x 75 and four conversions.
+//   A = 1/r + k/r^3, B = 1/r^3 - 3k/r^5, A'/r = B - 2/r^3, B'/r = (2/r^3 - 5 B) / r^2, k = c3/c1.
+template <int TENSOR, bool PER, bool SYM = true>
+__device__ __forceinline__ void vjp_sym_f64(const double (&t)[9], const double (&s)[9], const PairConst &c,
+                                            double (&M)[3], double (&G)[3], double (&JM)[3], double (&JG)[3]) {
+    double d[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        d[k] = __dsub_rn(t[k], s[k]);
+        if (PER) d[k] = min_image_f64(d[k], c.Ld[k], c.invLd[k]);
+    }
+    double r2 = __fma_rn(d[2], d[2], __fma_rn(d[1], d[1], __dmul_rn(d[0], d[0])));
+    r2 = less_pos64(r2, c.r2min_d) ? c.r2min_d : r2;
+    const double ri = rsqrt_int64(r2), ri2 = __dmul_rn(ri, ri), ri3 = __dmul_rn(ri, ri2);
     double A, B, dA, dB;
     if (TENSOR == T_OSEEN) {
-        A = c.c1_d * ri;
-        B = c.c1_d * ri3;
-        dA = -c.c1_d * ri3;
-        dB = -3.0 * c.c1_d * ri5;
+        A = ri;
+        B = ri3;
+        dA = -ri3;
+        dB = __dmul_rn(-3.0, __dmul_rn(ri3, ri2));
     } else {
-        A = ri * fma(c.c3_d, ri2, c.c1_d);
-        B = ri3 * fma(c.m3c3_d, ri2, c.c1_d);
-        dA = ri3 * fma(c.m3c3_d, ri2, -c.c1_d);
-        dB = ri5 * fma(-5.0 * c.m3c3_d, ri2, -3.0 * c.c1_d);
+        const double two = __dadd_rn(ri3, ri3);
+        A = __fma_rn(c.k_d, ri3, ri);
+        B = __fma_rn(c.m3k_d, __dmul_rn(ri3, ri2), ri3);
+        dA = __dsub_rn(B, two);
+        dB = __dmul_rn(ri2, __fma_rn(-5.0, B, two));
     }
-    const double Wir = dx * Wi.x + dy * Wi.y + dz * Wi.z;
-    const double Fir = dx * Fi.x + dy * Fi.y + dz * Fi.z;
-    const double Wjr = dx * w.x + dy * w.y + dz * w.z;
-    const double Fjr = dx * f.x + dy * f.y + dz * f.z;
-    const double U = Wi.x * f.x + Wi.y * f.y + Wi.z * f.z + w.x * Fi.x + w.y * Fi.y + w.z * Fi.z;
-    const double Q = Wir * Fjr + Wjr * Fir;
-    const double cr = dA * U + dB * Q;
-    const double bFj = B * Fjr, bWi = B * Wir, bFi = B * Fir, bWj = B * Wjr;
-    g.x += cr * dx + Wi.x * bFj + f.x * bWi + w.x * bFi + Fi.x * bWj;
-    g.y += cr * dy + Wi.y * bFj + f.y * bWi + w.y * bFi + Fi.y * bWj;
-    g.z += cr * dz + Wi.z * bFj + f.z * bWi + w.z * bFi + Fi.z * bWj;
-    m.x += A * w.x + bWj * dx;
-    m.y += A * w.y + bWj * dy;
-    m.z += A * w.z + bWj * dz;
+    auto dot = [](double a0, double a1, double a2, double b0, double b1, double b2) {
+        return __fma_rn(a2, b2, __fma_rn(a1, b1, __dmul_rn(a0, b0)));
+    };
+    const double Wir = dot(d[0], d[1], d[2], t[6], t[7], t[8]), Fir = dot(d[0], d[1], d[2], t[3], t[4], t[5]);
+    const double Wjr = dot(d[0], d[1], d[2], s[6], s[7], s[8]), Fjr = dot(d[0], d[1], d[2], s[3], s[4], s[5]);
+    const double U = __fma_rn(s[8], t[5], __fma_rn(s[7], t[4], __fma_rn(s[6], t[3],
+                              dot(t[6], t[7], t[8], s[3], s[4], s[5]))));
+    const double cr = __fma_rn(dB, __fma_rn(Wjr, Fir, __dmul_rn(Wir, Fjr)), __dmul_rn(dA, U));
+    const double bFj = __dmul_rn(B, Fjr), bWi = __dmul_rn(B, Wir), bFi = __dmul_rn(B, Fir), bWj = __dmul_rn(B, Wjr);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const double g = __fma_rn(cr, d[k], __fma_rn(t[6 + k], bFj, __fma_rn(s[3 + k], bWi, __fma_rn(s[6 + k], bFi,
+                                  __dmul_rn(t[3 + k], bWj)))));
+        G[k] = __dadd_rn(G[k], g);
+        M[k] = __fma_rn(bWj, d[k], __fma_rn(A, s[6 + k], M[k]));
+        if (SYM) {
+            JG[k] = __dsub_rn(JG[k], g);
+            JM[k] = __fma_rn(bWi, d[k], __fma_rn(A, t[6 + k], JM[k]));
+        }
+    }
 }
 
 // ---------------------------------------------------------------- compensated sums

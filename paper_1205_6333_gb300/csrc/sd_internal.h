@@ -382,9 +382,19 @@ cudaError_t launch_small(sd_handle *h, cudaStream_t st, int out, double *x0, dou
 cudaError_t vjp_setup(sd_handle *h);
 cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm, double *partM,
                              double *partG);
-cudaError_t launch_vjp_epilogue(sd_handle *h, cudaStream_t st, const double *x64, const void *posm,
-                                const double *F64, const void *frcm, const double *W64, const void *wm,
-                                int out_dtype, void *gx_out, void *gF_out, double dt, double *lam_acc,
-                                double *gF_acc);
+// What a vector-Jacobian product is taken of: positions (mirror: posm), forces, cotangents
+// (mirror: wam), and whose candidate list holds the near pairs (vlist: the Verlet steps').
+struct VjpInput {
+    const double *x64;
+    const double *F64;
+    Mirror frcm;
+    const double *W64;
+    bool vlist;
+};
+// The FP64 terms of the listed pairs (beside or before the all-pairs kernel), then the sums
+// and the results; out_dtype -1: lam_out = W + dt gX (mirror: wam), gF_acc += dt mu W.
+cudaError_t launch_vjp_near(sd_handle *h, cudaStream_t st, const VjpInput &in);
+cudaError_t launch_vjp_epilogue(sd_handle *h, cudaStream_t st, const VjpInput &in, int out_dtype, void *gx_out,
+                                void *gF_out, double dt, double *lam_out, double *gF_acc);
 
 }  // namespace sd
