@@ -400,13 +400,14 @@ __global__ void __launch_bounds__(kNT) dense2_kernel(const float *__restrict__ p
 // A pair in an off-diagonal tile is clamped iff the near pass raised the flag,
 // exactly as in dense2_kernel, and each direction's FP32 term is bit-identical to
 // dense2_kernel's; only the order of the sums differs.
-#ifndef SD_SYM_UNROLL
-#define SD_SYM_UNROLL 4
-#endif
+// Unroll of the packet loop: eight steps with four targets per lane (N = 65,536 / 131,072,
+// whole call: 2,287 / 8,763 us with four, 2,254 / 8,627 with eight; 16 outgrow the
+// instruction cache, 2,289 / 8,736), four with two (a step at N = 4,096 loses 1% with eight).
+template <int R>
+constexpr int kSymUnroll = R >= 4 ? 8 : 4;
 #ifndef SD_SYM_MINB
 #define SD_SYM_MINB 1
 #endif
-constexpr int kSymUnroll = SD_SYM_UNROLL;
 
 template <int TENSOR, bool CLAMP, bool PER, int R, int B>
 __device__ __forceinline__ void sym_tile(const f2 *__restrict__ sp, int lane, const f2 (&XI)[R], const f2 (&YI)[R],
@@ -414,12 +415,13 @@ __device__ __forceinline__ void sym_tile(const f2 *__restrict__ sp, int lane, co
                                          const PairConst2 &c, f2 (&AX)[R], f2 (&AY)[R], f2 (&AZ)[R],
                                          float *__restrict__ jw) {
     constexpr int S = B / 2;   // packets per array
+    constexpr int kUnroll = kSymUnroll<R>;
     const int nxt = (lane + 1) & 31;
 #pragma unroll 1
     for (int g = 0; g < B / 64; ++g) {
         const f2 *gp = sp + g * 32;
         f2 JX = 0ull, JY = 0ull, JZ = 0ull;
-#pragma unroll kSymUnroll
+#pragma unroll kUnroll
         for (int m = 0; m < 32; ++m) {
             const int p = (lane + m) & 31;
             const f2 PX = gp[p], PY = gp[S + p], PZ = gp[2 * S + p];

@@ -40,15 +40,17 @@ struct PairConst {
 };
 
 // Nearest image of a separation d in a dimension of period L (1/L = invL):
-// d - L rint(d / L), with rint(t) = (t + 1.5 2^23) - 1.5 2^23, exact round-to-even
-// for |t| < 2^22 (FP32; 2^51 for FP64).  The result is odd in d, bit for bit, so
+// d - L rint(d / L), with rint(d / L) = (d / L + 1.5 2^23) - 1.5 2^23, the sum in one
+// fused operation: exact round-to-even for |d / L| < 2^22 (FP32; 2^51 for FP64), three
+// operations a dimension (with the product apart, four: 482 -> 445 us for the FP64 product in
+// a box at N = 3,000).  The result is odd in d, bit for bit, so
 // the image of r_j - r_i is the negated image of r_i - r_j; with invL = 0 it is d.
 __device__ __forceinline__ float min_image_f32(float d, float L, float invL) {
-    const float n = __fsub_rn(__fadd_rn(__fmul_rn(d, invL), 12582912.0f), 12582912.0f);
+    const float n = __fsub_rn(__fmaf_rn(d, invL, 12582912.0f), 12582912.0f);
     return __fmaf_rn(-L, n, d);
 }
 __device__ __forceinline__ double min_image_f64(double d, double L, double invL) {
-    const double n = __dsub_rn(__dadd_rn(__dmul_rn(d, invL), 6755399441055744.0), 6755399441055744.0);
+    const double n = __dsub_rn(__fma_rn(d, invL, 6755399441055744.0), 6755399441055744.0);
     return __fma_rn(-L, n, d);
 }
 
@@ -157,7 +159,7 @@ inline PairConst2 pair_const2(const PairConst &pc, int n) {
 
 __device__ __forceinline__ f2 min_image2(f2 d, f2 negL, f2 invL) {
     const f2 magic = 0x4B4000004B400000ull;   // (1.5 2^23, 1.5 2^23)
-    const f2 n = sub2(add2(mul2(d, invL), magic), magic);
+    const f2 n = sub2(fma2(d, invL, magic), magic);
     return fma2(negL, n, d);
 }
 
@@ -412,55 +414,9 @@ __device__ __forceinline__ void profile_exact(double r2, const PairConst &c, dou
 //   m += A Wj + B (r.Wj) r                                  (row i of mu W)
 //   g += (dA U + dB Q) r + B [Wi (Fj.r) + Fj (Wi.r) + Wj (Fi.r) + Fi (Wj.r)]
 // with U = Wi.Fj + Wj.Fi and Q = (Wi.r)(Fj.r) + (Wj.r)(Fi.r)  -- the gradient of
-// Wi.T(r)Fj + Wj.T(r)Fi with respect to x_i.  FP32, r^2 clamped like pair_f32.
-template <int TENSOR, bool PER = false>
-__device__ __forceinline__ void vjp_pair_f32(float xi, float yi, float zi, float3 Fi, float3 Wi, float4 p, float4 f,
-                                             float4 w, const PairConst &c, float3 &m, float3 &g) {
-    float dx = __fsub_rn(xi, p.x);
-    float dy = __fsub_rn(yi, p.y);
-    float dz = __fsub_rn(zi, p.z);
-    if (PER) {
-        dx = min_image_f32(dx, c.Lf[0], c.invLf[0]);
-        dy = min_image_f32(dy, c.Lf[1], c.invLf[1]);
-        dz = min_image_f32(dz, c.Lf[2], c.invLf[2]);
-    }
-    float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-    r2 = fmaxf(r2, c.r2min_f);
-    const float ri = rsqrt_sfu(r2);
-    const float ri2 = __fmul_rn(ri, ri);
-    const float ri3 = __fmul_rn(ri, ri2);
-    const float ri5 = __fmul_rn(ri3, ri2);
-    float A, B, dA, dB;
-    if (TENSOR == T_OSEEN) {
-        A = __fmul_rn(c.c1_f, ri);
-        B = __fmul_rn(c.c1_f, ri3);
-        dA = __fmul_rn(-c.c1_f, ri3);
-        dB = __fmul_rn(-3.0f * c.c1_f, ri5);
-    } else {
-        A = __fmul_rn(ri, __fmaf_rn(c.c3_f, ri2, c.c1_f));
-        B = __fmul_rn(ri3, __fmaf_rn(c.m3c3_f, ri2, c.c1_f));
-        dA = __fmul_rn(ri3, __fmaf_rn(c.m3c3_f, ri2, -c.c1_f));                 // -c1/r^3 - 3c3/r^5
-        dB = __fmul_rn(ri5, __fmaf_rn(-5.0f * c.m3c3_f, ri2, -3.0f * c.c1_f));  // -3c1/r^5 + 15c3/r^7
-    }
-    const float Wir = __fmaf_rn(dz, Wi.z, __fmaf_rn(dy, Wi.y, __fmul_rn(dx, Wi.x)));
-    const float Fir = __fmaf_rn(dz, Fi.z, __fmaf_rn(dy, Fi.y, __fmul_rn(dx, Fi.x)));
-    const float Wjr = __fmaf_rn(dz, w.z, __fmaf_rn(dy, w.y, __fmul_rn(dx, w.x)));
-    const float Fjr = __fmaf_rn(dz, f.z, __fmaf_rn(dy, f.y, __fmul_rn(dx, f.x)));
-    const float WiFj = __fmaf_rn(Wi.z, f.z, __fmaf_rn(Wi.y, f.y, __fmul_rn(Wi.x, f.x)));
-    const float U = __fmaf_rn(w.z, Fi.z, __fmaf_rn(w.y, Fi.y, __fmaf_rn(w.x, Fi.x, WiFj)));
-    const float Q = __fmaf_rn(Wjr, Fir, __fmul_rn(Wir, Fjr));
-    const float cr = __fmaf_rn(dB, Q, __fmul_rn(dA, U));
-    const float bFj = __fmul_rn(B, Fjr), bWi = __fmul_rn(B, Wir), bFi = __fmul_rn(B, Fir), bWj = __fmul_rn(B, Wjr);
-    g.x = __fmaf_rn(cr, dx, __fmaf_rn(Wi.x, bFj, __fmaf_rn(f.x, bWi, __fmaf_rn(w.x, bFi, __fmaf_rn(Fi.x, bWj, g.x)))));
-    g.y = __fmaf_rn(cr, dy, __fmaf_rn(Wi.y, bFj, __fmaf_rn(f.y, bWi, __fmaf_rn(w.y, bFi, __fmaf_rn(Fi.y, bWj, g.y)))));
-    g.z = __fmaf_rn(cr, dz, __fmaf_rn(Wi.z, bFj, __fmaf_rn(f.z, bWi, __fmaf_rn(w.z, bFi, __fmaf_rn(Fi.z, bWj, g.z)))));
-    m.x = __fmaf_rn(bWj, dx, __fmaf_rn(A, w.x, m.x));
-    m.y = __fmaf_rn(bWj, dy, __fmaf_rn(A, w.y, m.y));
-    m.z = __fmaf_rn(bWj, dz, __fmaf_rn(A, w.z, m.z));
-}
-
-// Packed constants of vjp_pair_f32x2: the values vjp_pair_f32 forms from PairConst,
-// each as a (c, c) pair (products such as -5 m3c3 rounded in FP32 as there).
+// Wi.T(r)Fj + Wj.T(r)Fi with respect to x_i.
+//
+// Packed constants of the FP32 pair terms, each as a (c, c) pair.
 struct VjpConst2 {
     f2 c1, c3, m3c3, nc1, n5m3c3, n3c1;   // c1, c3, m3c3, -c1, -5 m3c3, -3 c1
     float r2min;
@@ -468,9 +424,8 @@ struct VjpConst2 {
 };
 
 // Two pairs at once, (i, j0) and (i, j1): XI.. FI.. WI.. = the target's values in both
-// lanes, P* F* W* = (source j0, source j1).  Lane by lane the operation sequence of
-// vjp_pair_f32, so each lane's terms are bit-identical to it (the epilogue subtracts
-// vjp_pair_f32's value for the pairs closer than r_near).
+// lanes, P* F* W* = (source j0, source j1); r^2 clamped like pair_f32.  (The near terms are
+// taken out of the sums by evaluating the same function on the same operands.)
 template <int TENSOR, bool PER = false>
 __device__ __forceinline__ void vjp_pair_f32x2(f2 XI, f2 YI, f2 ZI, f2 FIx, f2 FIy, f2 FIz, f2 WIx, f2 WIy, f2 WIz,
                                                f2 PX, f2 PY, f2 PZ, f2 FX, f2 FY, f2 FZ, f2 WX, f2 WY, f2 WZ,

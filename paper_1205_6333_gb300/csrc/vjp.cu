@@ -313,8 +313,8 @@ __device__ __forceinline__ void sym_tile_at(const DenseGeom &g, long long t, int
 // not fit the registers), walked as in dense_sym_kernel; diagonal tiles run the directed
 // pair.  Target sums are folded into (hi, lo) sums after every 64 sources; a tile's source sums
 // are added over the warps in fixed order and go to its own rows of jpart in FP32.
-// N = 4,096: 42 us directed, 31 (55% of the pipe: 3.5 CTAs of two warps an SM; one target per
-// lane and four warps are slower, 34); whole call at 4,096 / 16,384: 96 / 716 -> 57 / 393 us.
+// N = 4,096: 42 us directed, 31 (55% of the pipe: 3.5 CTAs of two warps an SM); whole call at
+// 4,096 / 16,384: 96 / 716 -> 57 / 393 us (with one target per lane and four warps 59 at 4,096).
 template <int TENSOR, bool PER, int B, int NT>
 __global__ void __launch_bounds__(NT) vjp_sym_kernel(const float *__restrict__ pos, const float *__restrict__ frc,
                                                      const float *__restrict__ wv, double *__restrict__ partM,
