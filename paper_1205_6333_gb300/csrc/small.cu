@@ -5,7 +5,7 @@
 // (check, list rebuild, near pass, all-pairs kernel, epilogue) and of dependent loads and
 // FP64 operations in each: N = 1,021 has 0.6 us of FP32 work per step on the whole chip
 // and took 25 us through those kernels, four spheres in FP64 80 us, set_positions and one
-// product at N = 1,000 106 us.  Through this one: 6.8 us, 2.7 us and 24 us (about half of
+// product at N = 1,000 106 us.  Through this one: 6.8 us, 2.6 us and 24 us (about half of
 // it the host's two calls).
 // Here a step is two phases of one kernel:
 //   A  a thread-block cluster takes a block of targets, its CTAs the j-splits; each sums
@@ -185,8 +185,11 @@ __device__ __noinline__ bool small_near(const SmallArgs &a, const SmallNear &m, 
     return true;
 }
 
-// One pair of the FP64 sum.  Closer than 2a: the self pair adds nothing (its term
-// mu_ii / mu0 = I joins in phase B), an overlapping pair its exact term.
+// One pair of the FP64 sum, divided by c1 (phase B multiplies the sums).  Closer than 2a: the
+// self pair adds nothing (its term mu_ii / mu0 = I joins in phase B), an overlapping pair its
+// exact term.  25 FP64 operations, no conversions and no FP64 comparison: they bound the
+// larger systems (two a clock and SM), and their chain the smallest
+// (with them the product at n = 1,000 75 us, 512 steps of four spheres 1.39 ms; now 63 and 1.31).
 template <int TENSOR, bool PER>
 __device__ __forceinline__ void small_pair64(double xi, double yi, double zi, double px, double py, double pz, double fx,
                                              double fy, double fz, bool self, const SmallArgs &a, double &ax,
@@ -199,7 +202,7 @@ __device__ __forceinline__ void small_pair64(double xi, double yi, double zi, do
     }
     const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
     double A, B;
-    if (r2 < a.pc.r2min_d) {
+    if (less_pos64(r2, a.pc.r2min_d)) {
         if (self) return;
         if (r2 == 0.0 && TENSOR != T_RPY) {
             atomicOr(a.err, DEV_ERR_COINCIDENT);
@@ -207,15 +210,10 @@ __device__ __forceinline__ void small_pair64(double xi, double yi, double zi, do
         }
         double dA, dB;
         profile_exact<TENSOR>(r2, a.pc, A, B, dA, dB);
+        A *= a.pc.invc1_d;
+        B *= a.pc.invc1_d;
     } else {
-        const double ri = rsqrt_nr64(r2), ri2 = __dmul_rn(ri, ri);
-        if (TENSOR == T_OSEEN) {
-            A = __dmul_rn(a.pc.c1_d, ri);
-            B = __dmul_rn(A, ri2);
-        } else {
-            A = __dmul_rn(ri, __fma_rn(a.pc.c3_d, ri2, a.pc.c1_d));
-            B = __dmul_rn(__dmul_rn(ri, ri2), __fma_rn(a.pc.m3c3_d, ri2, a.pc.c1_d));
-        }
+        profile64<TENSOR>(r2, a.pc, A, B);
     }
     const double s = __dmul_rn(B, __fma_rn(dz, fz, __fma_rn(dy, fy, __dmul_rn(dx, fx))));
     ax = __fma_rn(s, dx, __fma_rn(A, fx, ax));
@@ -570,7 +568,9 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
         } else if (upd) {
             double v = self;
             if constexpr (MODE == MODE_FP64) {
-                for (int s = 0; s < a.nsplit; ++s) v += s_v[(s * 3 + ed) * a.rows + er];
+                double sum = s_v[ed * a.rows + er];
+                for (int s = 1; s < a.nsplit; ++s) sum += s_v[(s * 3 + ed) * a.rows + er];
+                v = __fma_rn(a.pc.c1_d, sum, v);
             } else {
                 const float2 *q = reinterpret_cast<const float2 *>(s_v) + ed * a.rows + er;
                 float h = q[0].x, l = q[0].y;
