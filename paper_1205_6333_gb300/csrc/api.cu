@@ -735,10 +735,15 @@ static sd_status ensure_cells(sd_handle *h) {
 static cudaError_t near_list(sd_handle *h, bool vjp) {
     const double *x = h->x64[h->cur];
     if (h->cells_valid && vjp && h->near_valid) return cudaSuccess;
-    h->near_valid = true;
-    if (h->cells_valid) return launch_near_collect(h, h->stream, x, h->posm.aos, h->Fa64, h->frcam.aos, false);
-    const cudaError_t e = launch_near_lists(h, h->stream, x, h->posm, h->Fa64, h->frcam.aos);
-    h->cells_valid = e == cudaSuccess;
+    h->near_valid = false;
+    cudaError_t e;
+    if (h->cells_valid) {
+        e = launch_near_collect(h, h->stream, x, h->posm.aos, h->Fa64, h->frcam.aos, false);
+    } else {
+        e = launch_near_lists(h, h->stream, x, h->posm, h->Fa64, h->frcam.aos);
+        h->cells_valid = e == cudaSuccess;
+    }
+    h->near_valid = e == cudaSuccess;
     return e;
 }
 
