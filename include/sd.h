@@ -122,8 +122,8 @@ typedef struct sd_config {
                                 (SD_ERR_UNSUPPORTED). */
     double verlet_skin;      /* neighbour-list skin of sd_step (Sec. 3.1 step 2, Verlet lists): 0 = default
                                 0.5a, < 0 = off.  The steps keep an FP64 near-pair list of the pairs
-                                within its cutoff + skin, built by sd_set_positions and rebuilt once some
-                                particle has moved skin / 4 relative to particle 0 since the last
+                                within its cutoff + skin, built by the first step after sd_set_positions
+                                and rebuilt once some particle has moved skin / 4 relative to particle 0 since the last
                                 build (a uniform translation never forces one; up to skin / 2 the
                                 list still holds every pair within its cutoff, the largest of r_near,
                                 rep_rc with repulsion and 3a with lubrication).  With constant forces
@@ -237,8 +237,9 @@ sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, 
  *   lambda_T = gxT;  lambda_n = lambda_{n+1} + dt (dv/dx(x_n))^T lambda_{n+1};
  *   gx0 = lambda_0;  gF = dL/dF_ext = sum_n dt mu(x_n) lambda_{n+1}.
  * The forward pass is re-run with FP64 checkpoints every ckpt_every steps
- * (ckpt_every >= 1) and each segment is recomputed once.  The handle's positions
- * are restored to x0 on return.  gxT input, gx0 and gF outputs (n x 3 doubles). */
+ * (ckpt_every >= 1) and each segment is recomputed once; while the positions of all
+ * steps take at most 256 MB (and the memory is there) they are kept instead, and
+ * nothing is recomputed.  The handle's positions are restored to x0 on return.  gxT input, gx0 and gF outputs (n x 3 doubles). */
 sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every, const double *gxT, double *gx0,
                      double *gF, int on_device);
 

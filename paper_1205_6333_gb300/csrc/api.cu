@@ -335,6 +335,10 @@ static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int
     return e;
 }
 
+// Up to this many bytes sd_adjoint keeps the positions of all steps; beyond, checkpoints.
+// (N = 4,096, 40 steps in segments of 20: 3,892 us with two segments recomputed, 3,345 so.)
+constexpr double kKeepBytes = 256.0 * 1024 * 1024;
+
 // Graphs of both parts for a full segment of K steps (the recompute part only when
 // K > 1), cached per (dt, K).
 static sd_status capture_adjoint(sd_handle *h, double dt, int64_t K) {
@@ -1090,15 +1094,20 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
     const size_t mb = static_cast<size_t>(h->npad) * v4size(h);
     const int64_t K = ckpt_every;
     const int64_t nck = nsteps / K + 1;
-    // storage: checkpoints, one segment of positions + mirrors, lambda, gF accumulator
-    const size_t ck_need = static_cast<size_t>(nck) * xb;
-    if (!h->ckpt || h->ckpt_bytes < ck_need) {
+    // storage: the positions of every step while they are few (nothing is then recomputed),
+    // else checkpoints; one segment of positions, lambda, gF accumulator
+    auto store = [&](size_t need) {
+        if (h->ckpt && h->ckpt_bytes >= need) return true;
         dfree(h, h->ckpt);
-        h->ckpt = static_cast<double *>(dalloc(h, ck_need));
-        h->ckpt_bytes = h->ckpt ? ck_need : 0;
-        if (!h->ckpt) return set_error(SD_ERR_OOM, "device allocation of checkpoints");
-    }
-    const size_t seg_need = static_cast<size_t>(K) * xb;
+        h->ckpt = static_cast<double *>(dalloc(h, need));
+        h->ckpt_bytes = h->ckpt ? need : 0;
+        return h->ckpt != nullptr;
+    };
+    const bool keep = nsteps > 0 && static_cast<double>(nsteps) * xb <= kKeepBytes && store(static_cast<size_t>(nsteps) * xb);
+    if (!keep && !store(static_cast<size_t>(nck) * xb))
+        return set_error(SD_ERR_OOM, "device allocation of checkpoints");
+    const bool small = use_small(h);
+    const size_t seg_need = (static_cast<size_t>(K) + (keep && !small ? 1 : 0)) * xb;
     {
         sd_status s0 = ensure_seg(h, seg_need, "device allocation of the recompute segment");
         if (s0 != SD_OK) return s0;
@@ -1111,15 +1120,56 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
 
     const int c0 = h->cur;
     const int64_t nseg = (nsteps + K - 1) / K;
-    // forward with checkpoints, segment by segment through the step graphs (the state
-    // ping-pongs through x64[0], x64[1])
-    SD_CUDA(cudaMemcpyAsync(h->ckpt, h->x64[c0], xb, cudaMemcpyDeviceToDevice, st));
-    // (the last segment's steps are those that its recompute takes: x_T itself is not needed)
+    auto kept = [&](int64_t k) { return h->ckpt + static_cast<size_t>(k) * n3; };   // x_k, or checkpoint k
+    auto copy_x = [&](double *to, const double *from, int64_t k) {
+        return cudaMemcpyAsync(to, from, static_cast<size_t>(k) * xb, cudaMemcpyDeviceToDevice, st);
+    };
+    h->cells_valid = false;
     if (h->verlet && !h->list_set) {
         sd_status ss = build_list(h);
         if (ss != SD_OK) return ss;
     }
-    for (int64_t sg = 0; sg + 1 < nseg; ++sg) {
+    // Steps within a segment of positions in seg: the cached graph of a full one, eager
+    // launches with the profiler on and for a shorter last one.
+    auto segment = [&](int64_t len, int part) -> sd_status {
+        if (len != K || h->prof.on)
+            return launch_check(adjoint_segment(h, st, dt, len, part), part ? "adjoint sweep" : "recompute");
+        if (!h->adj_rev || h->adj_dt != dt || h->adj_K != K) {
+            sd_status ss = capture_adjoint(h, dt, K);
+            if (ss != SD_OK) return ss;
+        }
+        cudaGraphExec_t g = part ? h->adj_rev : h->adj_rec;
+        if (g) {
+            SD_CUDA(cudaGraphLaunch(g, st));
+            h->launches += part ? h->adj_rev_kernels : h->adj_rec_kernels;
+        }
+        return SD_OK;
+    };
+    // forward, up to x_{T-1} (x_T itself is not needed)
+    if (keep && small) {
+        SD_CUDA(copy_x(kept(0), h->x64[c0], 1));
+        if (nsteps > 1) {
+            sd_status ss = launch_check(launch_small(h, st, OUT_EULER, kept(0), nullptr, n3, h->F64, 0, nullptr, dt,
+                                                     nsteps - 1, 0, h->n),
+                                        "forward steps");
+            if (ss != SD_OK) return ss;
+        }
+    } else if (keep) {
+        SD_CUDA(copy_x(segx(0), h->x64[c0], 1));
+        for (int64_t sg = 0; sg < nseg; ++sg) {
+            sd_status ss = segment(std::min(K, nsteps - sg * K), 0);
+            if (ss == SD_OK && sg + 1 < nseg)   // on to the next segment's first positions
+                ss = launch_check(launch_step(h, st, dt, segx(K - 1), segx(K)), "forward step");
+            if (ss != SD_OK) return ss;
+            if (sg + 1 < nseg) {   // (the last segment stays in seg)
+                SD_CUDA(copy_x(kept(sg * K), segx(0), K));
+                SD_CUDA(copy_x(segx(0), segx(K), 1));
+            }
+        }
+    } else {   // with checkpoints, through the step graphs (the state ping-pongs through x64[0], x64[1])
+        SD_CUDA(copy_x(h->ckpt, h->x64[c0], 1));
+    }
+    for (int64_t sg = 0; !keep && sg + 1 < nseg; ++sg) {   // (the last segment's steps are its recompute's)
         const int64_t len = std::min(K, nsteps - sg * K);
         sd_status ss = run_steps(h, dt, len);
         if (ss != SD_OK) return ss;
@@ -1138,31 +1188,22 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
         sd_status ss = launch_check(launch_stage_forces(h, st, h->lam, SD_DTYPE_F64, 0, h->Wa64, h->wam), "stage lambda");
         if (ss != SD_OK) return ss;
     }
-    // reverse sweep, last segment first: recompute the segment's positions from its
-    // checkpoint, then walk it backwards.  Full segments replay cached graphs (eager
-    // with the profiler on, and for a shorter last segment).
+    // reverse sweep, last segment first: take the segment's positions from what was kept, or
+    // recompute them from its checkpoint, then walk it backwards
     for (int64_t sg = nseg - 1; sg >= 0; --sg) {
         const int64_t len = std::min(K, nsteps - sg * K);
-        SD_CUDA(cudaMemcpyAsync(segx(0), h->ckpt + static_cast<size_t>(sg) * n3, xb, cudaMemcpyDeviceToDevice, st));
-        if (len == K && !h->prof.on) {
-            if (!h->adj_rev || h->adj_dt != dt || h->adj_K != K) {
-                sd_status ss = capture_adjoint(h, dt, K);
-                if (ss != SD_OK) return ss;
-            }
-            if (h->adj_rec) {
-                SD_CUDA(cudaGraphLaunch(h->adj_rec, st));
-                h->launches += h->adj_rec_kernels;
-            }
-            SD_CUDA(cudaGraphLaunch(h->adj_rev, st));
-            h->launches += h->adj_rev_kernels;
+        sd_status ss = SD_OK;
+        if (keep) {
+            if (small || sg + 1 < nseg) SD_CUDA(copy_x(segx(0), kept(sg * K), len));
         } else {
-            sd_status ss = launch_check(adjoint_segment(h, st, dt, len, 0), "recompute");
-            if (ss == SD_OK) ss = launch_check(adjoint_segment(h, st, dt, len, 1), "adjoint sweep");
-            if (ss != SD_OK) return ss;
+            SD_CUDA(copy_x(segx(0), kept(sg), 1));
+            ss = segment(len, 0);
         }
+        if (ss == SD_OK) ss = segment(len, 1);
+        if (ss != SD_OK) return ss;
     }
     // restore x0 into the current buffers
-    SD_CUDA(cudaMemcpyAsync(h->x64[c0], h->ckpt, xb, cudaMemcpyDeviceToDevice, st));
+    if (!keep) SD_CUDA(copy_x(h->x64[c0], h->ckpt, 1));
     sd_status ss = launch_check(launch_stage_pos(h, st, h->x64[c0], h->posm), "restore positions");
     if (ss != SD_OK) return ss;
     h->cur = c0;
