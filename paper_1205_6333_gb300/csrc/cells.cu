@@ -546,9 +546,12 @@ __global__ void __launch_bounds__(64) forces_list_kernel(const double *__restric
     double sum[3] = {0.0, 0.0, 0.0};
     if (cnt < 0) {   // a particle the overflowed list corrects in place: the cell list (rebuilt
                      // every step while the list overflows) gives its pairs
-        if (sub == 0) for_each_neighbour_part(c, i, c.cell[i], 0, 1, pair);
-        for (int d = 0; d < 3; ++d) sum[d] = f[d];
+        for_each_neighbour_part(c, i, c.cell[i], sub, L, pair);
     }
+    if (__any_sync(0xffffffffu, cnt < 0))
+#pragma unroll
+        for (int l = 0; l < L; ++l)
+            for (int d = 0; d < 3; ++d) sum[d] += __shfl_sync(0xffffffffu, cnt < 0 ? f[d] : 0.0, l, L);
     const long long e0 = cnt > 0 ? dbg_index(noff[i], static_cast<long long>(cap) - cnt + 1, err) : 0;
     const int rounds = __reduce_max_sync(0xffffffffu, (max(cnt, 0) + L - 1) / L);
     for (int r = 0; r < rounds; ++r) {

@@ -416,9 +416,11 @@ cudaError_t launch_near_pairs(sd_handle *h, cudaStream_t st, const double *x64, 
     if (h->n == 0) return cudaSuccess;
     NearArgs a = near_args(h, x64, posm, F64, frcm, h->r_near, verlet_step);
     if (verlet_step) a.flag = nullptr;   // (the check kernel's; the all-pairs kernel may be reading it)
-    // two pairs a particle in one pass, any more in turn (CTAs that find no pair crowd the
-    // all-pairs kernel beside them)
-    const int np = static_cast<int>(std::min<long long>((2LL * h->n + 127) / 128, 8LL * h->num_sms));
+    // eight pairs a particle in one pass, any more in turn: a suspension has one or two, an fcc
+    // lattice 12 to 18 (two a pass made its step at N = 4,000 85 us instead of 44); at most
+    // two CTAs an SM, as CTAs that find no pair crowd the all-pairs kernel beside them
+    // (repulsion, N = 16,384: 1% with 1,024)
+    const int np = static_cast<int>(std::min<long long>((8LL * h->n + 127) / 128, 2LL * h->num_sms));
     SD_NEAR_DISPATCH(near_launch_pairs, np);
     ++h->launches;
     return cudaGetLastError();

@@ -45,6 +45,8 @@ constexpr int kSmWarps = 16;               // one CTA per SM; 16 warps share a b
 constexpr int kSmThreads = 32 * kSmWarps + 32;   // ... and one more takes the near pairs of the last step
 constexpr int kSmAhead = 64;               // near pairs evaluated ahead (more: after the loop, by all threads)
 constexpr int kSmNotes = 512;              // noted pairs a CTA holds; more: its targets scan their range again
+constexpr double kSmDense = 8192.0;        // expected near pairs (known in a box) from which the near pass's full warps
+                                           // win: an fcc lattice of 2,048 52 us a step here, 48 there; 864: 29 and 41
 constexpr int kSmSoloFP32 = 128;           // largest n one CTA takes (FP32C)
 constexpr int kSmSoloFP64 = 16;            // ... FP64: two FP64 operations a clock and SM, so more SMs sooner
 constexpr int kSmMaxSteps = 512;           // steps per launch
@@ -491,16 +493,47 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
                         else
                             small_near<TENSOR, PER>(a, nr, key, s_cor + 3 * rank);
                     }
-                } else {   // the notes overflowed: each target scans the CTA's sources again, in order
-                    for (int t = tid; t < nt; t += kSmThreads) {
+                } else {
+                    // The notes overflowed (a lattice whose indices follow its sites): four lanes
+                    // of each target scan the CTA's sources again, 32 each at a time, and take
+                    // the FP64 terms of those within reach together (a term at a time as they
+                    // are met: 0.18 ms a step for 108 spheres of an fcc lattice); the lanes meet
+                    // in a fixed tree.
+                    for (int t4 = tid; t4 < 4 * nt; t4 += kSmThreads) {   // (whole warps)
+                        const int t = t4 >> 2, sub = t4 & 3;
                         double sum[3] = {0.0, 0.0, 0.0};
-                        if (i0 + t < a.n)
-                            for (int q = 0; q < jn; ++q) {
-                                double c[3];
-                                if (j0 + q != i0 + t && small_near<TENSOR, PER>(a, nr, (t << 16) | q, c))
-                                    for (int d = 0; d < 3; ++d) sum[d] += c[d];
+                        for (int q0 = sub; q0 - sub < jn; q0 += 128) {
+                            unsigned hit = 0;
+                            for (int k = 0; k < 32; ++k) {
+                                const int q = q0 + 4 * k;
+                                if (q >= jn) break;
+                                float dx = __fsub_rn(s_tgt[t], s_src[q]), dy = __fsub_rn(s_tgt[nt + t], s_src[a.jlen + q]),
+                                      dz = __fsub_rn(s_tgt[2 * nt + t], s_src[2 * a.jlen + q]);
+                                if (PER) {
+                                    dx = min_image_f32(dx, a.pc.Lf[0], a.pc.invLf[0]);
+                                    dy = min_image_f32(dy, a.pc.Lf[1], a.pc.invLf[1]);
+                                    dz = min_image_f32(dz, a.pc.Lf[2], a.pc.invLf[2]);
+                                }
+                                if (__fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))) <= a.rscreen2 &&
+                                    j0 + q != i0 + t && i0 + t < a.n)
+                                    hit |= 1u << k;
                             }
-                        for (int d = 0; d < 3; ++d) s_cor[3 * t + d] = sum[d];   // (nt <= kSmNotes)
+                            while (__any_sync(0xffffffffu, hit != 0)) {
+                                if (hit) {
+                                    double c[3];
+                                    const int q = q0 + 4 * (__ffs(hit) - 1);
+                                    hit &= hit - 1;
+                                    if (small_near<TENSOR, PER>(a, nr, (t << 16) | q, c))
+                                        for (int d = 0; d < 3; ++d) sum[d] += c[d];
+                                }
+                                __syncwarp();
+                            }
+                        }
+                        for (int d = 0; d < 3; ++d) {
+                            sum[d] += __shfl_xor_sync(0xffffffffu, sum[d], 1);
+                            sum[d] += __shfl_xor_sync(0xffffffffu, sum[d], 2);
+                            if (sub == 0) s_cor[3 * t + d] = sum[d];   // (nt <= kSmNotes)
+                        }
                     }
                 }
             }
@@ -656,6 +689,13 @@ cudaError_t small_setup(sd_handle *h) {
     const bool f64 = h->mode == MODE_FP64;
     const int n = h->n;
     g.solo = n <= (f64 ? kSmSoloFP64 : kSmSoloFP32);
+    // (FP32C near pairs cost one SM some 900 cycles a warp of them: a dense box takes more SMs)
+    if (!f64 && h->pc.Ld[0] > 0.0 && h->pc.Ld[1] > 0.0 && h->pc.Ld[2] > 0.0) {
+        const double rn = h->r_near;
+        const double close = 4.18879 * rn * rn * rn * n / (h->pc.Ld[0] * h->pc.Ld[1] * h->pc.Ld[2]);
+        if (n * close > kSmNotes) g.solo = 0;
+        if (n * close > kSmDense) return cudaSuccess;
+    }
     if (f64)
         while (g.iw > 1 && g.iw / 2 >= n) g.iw /= 2;
     bool tried[3][kSmMaxSplit + 1] = {};
