@@ -899,7 +899,8 @@ cudaError_t dense_setup(sd_handle *h) {
     const int nreal = std::max(h->n, 1);
     g.nIB = (nreal + g.I - 1) / g.I;
     void *fn = pick_dense(h->tensor, h->mode, h->pc.periodic != 0);
-    const void *chosen = fn;
+    cudaError_t e = allow_smem(fn, h->dense_limit);
+    if (e != cudaSuccess) return e;
     const int Jcand[4] = {kJmax, 128, 64, 32};
     int occ = 0;
     for (int ci = 0; ci < 4; ++ci) {
@@ -907,8 +908,6 @@ cudaError_t dense_setup(sd_handle *h) {
         if (h->mode == MODE_FP64 && J > 128) continue;
         if (h->mode != MODE_FP64 && J < 64) continue;   // (32-source tiles: FP64 only)
         const size_t smem = dense_smem(h->mode, J);
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kNT, smem);
         if (e != cudaSuccess) return e;
         g.J = J;
@@ -942,8 +941,8 @@ cudaError_t dense_setup(sd_handle *h) {
                                                            : reinterpret_cast<void *>(&dense_sym64_kernel<T_OSEEN, false>))
                                          : (h->pc.periodic ? reinterpret_cast<void *>(&dense_sym64_kernel<T_RP, true>)
                                                            : reinterpret_cast<void *>(&dense_sym64_kernel<T_RP, false>));
-        cudaError_t e = cudaFuncSetAttribute(sfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(sym64_smem()));
+        size_t limit = 0;
+        e = allow_smem(sfn, limit);
         if (e != cudaSuccess) return e;
         int socc = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&socc, sfn, kB64, sym64_smem());
@@ -960,13 +959,13 @@ cudaError_t dense_setup(sd_handle *h) {
             g = s;
             occ = socc;
             h->sym_nt = kB64;
-            chosen = sfn;
+            h->dense_limit = limit;
         }
     }
     if (h->mode != MODE_FP64 && h->npad % B == 0 && want_sym != SD_DENSE_DIRECTED) {
         void *sfn = pick_sym(h->tensor, h->mode, h->pc.periodic != 0, B, NT);
-        cudaError_t e = cudaFuncSetAttribute(sfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(sym_smem(B, NT)));
+        size_t limit = 0;
+        e = allow_smem(sfn, limit);
         if (e != cudaSuccess) return e;
         int socc = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&socc, sfn, NT, sym_smem(B, NT));
@@ -986,11 +985,9 @@ cudaError_t dense_setup(sd_handle *h) {
             g = s;
             occ = socc;
             h->sym_nt = NT;
-            chosen = sfn;
+            h->dense_limit = limit;
         }
     }
-    cudaError_t ea = allow_smem(chosen, h->dense_limit);
-    if (ea != cudaSuccess) return ea;
     int ms = 0;
     for (int ib = 0; ib < g.nIB; ++ib) ms = std::max(ms, geom_last(g, ib) - geom_first(g, ib) + 1);
     g.maxSlots = ms;

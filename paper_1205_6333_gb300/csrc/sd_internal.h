@@ -188,7 +188,9 @@ inline size_t spread_smem(int num_sms, int grid, int occ, size_t need, size_t li
     const size_t s = ((228 * 1024 / (per + 1) - 1024) / 128 + 1) * 128;   // (an SM's 228 KB; 1 KB a CTA is the system's)
     return s < need ? need : (s < limit ? s : limit);
 }
-// The most dynamic shared memory a launch of fn can have, and the attribute that allows it.
+// The most dynamic shared memory a launch of fn can have, and the attribute that allows it.  The
+// attribute belongs to the function, which every handle of the process shares: all set-ups
+// write this same value and nothing else, so none takes away what an older handle's launches need.
 inline cudaError_t allow_smem(const void *fn, size_t &limit) {
     cudaFuncAttributes at{};
     cudaError_t e = cudaFuncGetAttributes(&at, fn);

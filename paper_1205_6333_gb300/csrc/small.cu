@@ -734,8 +734,10 @@ cudaError_t small_setup(sd_handle *h) {
         g.rows = (g.nbl * 32 * g.R + g.split - 1) / g.split;
         g.smem = small_smem(h->mode, g.R, g.jlen, g.nbl, g.wb, g.solo, n);
         const void *fn = small_fn(h);
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(g.smem));
+        size_t limit = 0;
+        e = allow_smem(fn, limit);
         if (e != cudaSuccess) return e;
+        if (g.smem > limit) continue;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute at[2];
         small_config(h, cfg, at, nullptr, false);

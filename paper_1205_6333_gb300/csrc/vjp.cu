@@ -652,20 +652,12 @@ cudaError_t vjp_setup(sd_handle *h) {
         g.I = g.J = B;
         g.nIB = g.nJT = (std::max(h->n, 1) + B - 1) / B;
         g.nT = static_cast<long long>(g.nIB) * (g.nIB + 1) / 2;
-        cudaError_t e;
-        if (mode == MODE_FP64) {
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pick_vjp_sym64(h, B), B, 0);
-        } else {
-            const size_t smem = vjp_sym_smem(B, B / 2);
-            e = cudaFuncSetAttribute(pick_vjp_sym(h, B), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     static_cast<int>(smem));
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, pick_vjp_sym(h, B), B / 2, smem);
-        }
-        if (e != cudaSuccess) return e;
-        if (e == cudaSuccess) e = allow_smem(mode == MODE_FP64 ? reinterpret_cast<const void *>(pick_vjp_sym64(h, B))
-                                                              : reinterpret_cast<const void *>(pick_vjp_sym(h, B)),
-                                             h->vjp_limit);
+        const void *fn = mode == MODE_FP64 ? reinterpret_cast<const void *>(pick_vjp_sym64(h, B))
+                                           : reinterpret_cast<const void *>(pick_vjp_sym(h, B));
+        cudaError_t e = allow_smem(fn, h->vjp_limit);
+        if (e == cudaSuccess)
+            e = mode == MODE_FP64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, B, 0)
+                                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, B / 2, vjp_sym_smem(B, B / 2));
         if (e != cudaSuccess) return e;
         occ = std::max(occ, 1);
         const long long resident = static_cast<long long>(h->num_sms) * occ;
@@ -675,13 +667,13 @@ cudaError_t vjp_setup(sd_handle *h) {
         g.nIB = h->npad / g.I;
         const void *fn = mode == MODE_FP64 ? reinterpret_cast<const void *>(pick_vjp64(h))
                                            : reinterpret_cast<const void *>(pick_vjp2(h));
+        cudaError_t e = allow_smem(fn, h->vjp_limit);
+        if (e != cudaSuccess) return e;
         const int Jc[4] = {kJmax, 128, 64, SD_VJP_JMIN};
         for (int ci = 0; ci < 4; ++ci) {
             const int J = Jc[ci];
             if (mode == MODE_FP64 && J > 128) continue;
             const size_t smem = vjp_smem(mode, J);
-            cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-            if (e != cudaSuccess) return e;
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kNT, smem);
             if (e != cudaSuccess) return e;
             g.J = J;
