@@ -213,8 +213,9 @@ cudaError_t launch_pad_mirror(sd_handle *h, cudaStream_t st, Mirror m) {
 
 // Bins particle i and writes its mirror (position relative to particle 0, in the
 // dense kernels' precision), so the mirror is a pure function of the FP64 state.  A
-// Verlet list's build (xref given) records the positions in xref instead and leaves
-// the mirror and the clamp flag to the step's check kernel.
+// Verlet list's build (xref given) records the positions in xref too and leaves the
+// clamp flag to the step's check kernel; it needs the mirror of these positions, since the
+// list's candidates are screened on it and no step may have written it since they moved.
 template <typename V4>
 __global__ void cells_hash_kernel(const double *__restrict__ x, int n, CellList c, V4 *__restrict__ m,
                                   float *__restrict__ soa, int npad, int *flag, unsigned long long *near_n,
@@ -231,10 +232,9 @@ __global__ void cells_hash_kernel(const double *__restrict__ x, int n, CellList 
         xref[3 * i] = px;
         xref[3 * i + 1] = py;
         xref[3 * i + 2] = pz;
-    } else {
-        if (!isfinite(px) || !isfinite(py) || !isfinite(pz)) atomicOr(err, DEV_ERR_NONFINITE);
-        put_pos_mirror(m, soa, npad, i, x, c.box);
     }
+    if (!isfinite(px) || !isfinite(py) || !isfinite(pz)) atomicOr(err, DEV_ERR_NONFINITE);
+    put_pos_mirror(m, soa, npad, i, x, c.box);
     bin_particle(c, i, px, py, pz);
 }
 

@@ -343,7 +343,7 @@ cudaError_t launch_stage_pos(sd_handle *h, cudaStream_t st, const double *x64, M
 cudaError_t launch_stage_forces(sd_handle *h, cudaStream_t st, const void *src, int src_dtype, int add_ext,
                                 double *dst64, Mirror dstm, const void *src2 = nullptr, double *dst2 = nullptr,
                                 Mirror dstm2 = Mirror{});
-// xref != nullptr: a Verlet list's build (copies x64 to xref; the mirror is the check's).
+// xref != nullptr: a Verlet list's build (copies x64 to xref; the clamp flag is the check's).
 cudaError_t launch_build_cells(sd_handle *h, cudaStream_t st, const double *x64, Mirror posm,
                                double *xref = nullptr);
 // The same in a Verlet step, if its check asked for it.
