@@ -90,6 +90,9 @@ __device__ __forceinline__ uint32_t cluster_addr(const void *p, int rank) {
 __device__ __forceinline__ void cluster_store(uint32_t p, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(p), "d"(v) : "memory");
 }
+__device__ __forceinline__ void cluster_store(uint32_t p, int v) {
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
+}
 
 // Write / read (polling, bounded) one exchanged FP64 value of the step `tag`.
 __device__ __forceinline__ void xch_put(ulonglong2 *p, double v, unsigned tag) {
@@ -253,7 +256,8 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
     constexpr int TD = (TENSOR == T_OSEEN) ? T_OSEEN : T_RP;
     constexpr int I = small_block<MODE, R>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int s_fail, s_cnt[2];
+    __shared__ int2 s_end;   // x: a wait ran out here; y: the step in which one did somewhere in the cluster
+    __shared__ int s_cnt[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nt = a.nbl * I;                      // targets of this CTA
     const int WB = a.wb;                           // warps per target block
@@ -281,7 +285,7 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
     unsigned tag = 0;
     if (!a.solo && a.out == OUT_EULER && a.nsteps > 1) tag = *reinterpret_cast<volatile unsigned *>(a.sync);
     if (tid == 0) {
-        s_fail = 0;
+        s_end = make_int2(0, 0x7fffffff);
         s_cnt[0] = s_cnt[1] = 0;
     }
 
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
                             u[d] = from[3 * static_cast<size_t>(p) + d];
                         }
                     } else if (!xch_get(a, xb, p, tag + step - 1, org, u)) {
-                        s_fail = 1;
+                        s_end.x = 1;
                     }
                     for (int d = 0; d < 3; ++d) {
                         u[d] -= org[d];
@@ -366,9 +370,18 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
             }
         }
         __syncthreads();
-        if (s_fail) break;
+        // A wait ran out here: the cluster has to leave together, since its peers store into
+        // this CTA's shared memory (padding rows too, which no wait stands for).  So every CTA
+        // is told the step before its barrier, this one only meets them there, and all leave at
+        // this place in the next step (y is then the same for all threads: who finds it set
+        // tells nobody, and one told in this very step goes on).
+        const int2 end = s_end;
+        if (end.y < step) break;
+        const bool lost = end.x != 0;
+        if (lost && tid < a.nsplit)
+            cluster_store(cluster_addr(reinterpret_cast<const char *>(&s_end) + sizeof(int), tid), step);
         const int nprev = step == 0 ? 0 : s_cnt[cur ^ 1];   // the last step's notes
-        if (mine) {
+        if (mine && !lost) {
             const SmallNear nr{reinterpret_cast<const float *>(s_src), reinterpret_cast<const float *>(s_tgt), s_pd,
                                a.jlen, nt, j0};
             if constexpr (MODE != MODE_FP64) {   // the last step's near pairs at the new positions
@@ -627,9 +640,8 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
             }
         }
     }
-    // (a CTA whose wait ran out may still be written to by its cluster's peers, whose next
-    // cluster barrier this one matches)
-    if (a.nsplit > 1) cluster_barrier();
+    // (no CTA stores into another's shared memory after the last step's cluster barrier, which all
+    // CTAs of the cluster have passed)
     if (!a.solo && passes > 1 && tid == 0) {   // the last CTA out: the next launch's tags are new ones
         __threadfence();
         if (atomicAdd(a.sync + 2, 1u) == gridDim.x - 1) {
