@@ -787,6 +787,12 @@ static sd_status apply_rows(sd_handle *h, const void *F, void *V, int dtype, int
     }
     const TileWin w = row_window(h, row0, row1);
     if (use_small(h)) {
+        // (the kernel reads F while it writes V: a product in place takes its forces from a copy)
+        const char *fb = static_cast<const char *>(Fd), *vb = static_cast<const char *>(Vd);
+        if (fb < vb + bytes_out && vb < fb + bytes_in) {
+            SD_CUDA(cudaMemcpyAsync(h->Fa64, Fd, bytes_in, cudaMemcpyDeviceToDevice, h->stream));
+            Fd = h->Fa64;
+        }
         sd_status s = launch_check(launch_small(h, h->stream, dtype == SD_DTYPE_F32 ? OUT_F32 : OUT_F64, h->x64[h->cur],
                                                 nullptr, 0, Fd, dtype == SD_DTYPE_F32, Vd, 0.0, 1, row0, row1),
                                    "mobility product");
