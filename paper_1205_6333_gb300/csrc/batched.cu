@@ -124,8 +124,10 @@ __device__ __forceinline__ void exact_pair(S dx, S dy, S dz, S fx, S fy, S fz, c
 // with directed pairs (1,000 clusters of 4 .. 256: 3.1 ms a step; this one 0.79).
 //   * The cluster's positions (relative to its first particle) and forces are staged as six
 //     FP64 arrays, padded to whole blocks of 32 with far-away, force-free slots.  The warps
-//     take the block pairs (p, q), p <= q, in turn; every warp adds what a tile gives both
-//     its blocks to sums of its own, and the warps' sums are added in ascending order.
+//     take the block pairs (p, q), p <= q, in turn.  What the u-th gives both its blocks goes to
+//     the sum u mod 4, in ascending u, and the four are added in order: the result does not
+//     depend on the number of warps, which the autotuner picks by timing.  (With a sum per warp
+//     it did.  More than four warps add in turns of four between block barriers.)
 //   * A tile (p, q), p < q: lane l holds target l of block q and meets source (l + m) mod 32
 //     of block p at step m; the source's running sum moves one lane down per step.  The
 //     last block is often partly filled: with w >= its particles a power of two, 32 / w
@@ -165,7 +167,8 @@ __device__ __forceinline__ void pair64_sym(const double (&t)[6], const double *_
     J[2] = __fma_rn(v, dz, __fma_rn(a, t[5], J[2]));
 }
 
-constexpr size_t batch64_smem(int warps) { return (6 + 3 * static_cast<size_t>(warps)) * kMaxCluster * sizeof(double); }
+constexpr int kSums64 = 4;   // sums a cluster has: the tiles u = v mod 4 add to the v-th, in ascending order
+constexpr size_t batch64_smem() { return (6 + 3 * static_cast<size_t>(kSums64)) * kMaxCluster * sizeof(double); }
 
 template <int TENSOR, int NW>
 __global__ void __launch_bounds__(32 * NW) batched64_kernel(BatchArgs a) {
@@ -173,8 +176,8 @@ __global__ void __launch_bounds__(32 * NW) batched64_kernel(BatchArgs a) {
     __shared__ int s_t;
     double *S = s_b64;                                     // [6][kMaxCluster]
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    double *SUM = S + 6 * kMaxCluster;                     // [NW][3][kMaxCluster]
-    double *mine = SUM + static_cast<size_t>(wid) * 3 * kMaxCluster;
+    double *SUM = S + 6 * kMaxCluster;                     // [kSums64][3][kMaxCluster]
+    double *mine = SUM + static_cast<size_t>(wid % kSums64) * 3 * kMaxCluster;
     const dbl4 *frcm = static_cast<const dbl4 *>(a.frcm);
     for (;;) {
         if (tid == 0) s_t = static_cast<int>(atomicAdd(a.ctr, 1ULL));
@@ -196,57 +199,72 @@ __global__ void __launch_bounds__(32 * NW) batched64_kernel(BatchArgs a) {
             }
             for (int d = 0; d < 6; ++d) S[d * kMaxCluster + p] = v[d];
         }
-        for (int p = lane; p < 32 * nb; p += 32)
-            for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + p] = 0.0;
+        if (wid < kSums64)
+            for (int p = lane; p < 32 * nb; p += 32)
+                for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + p] = 0.0;
         __syncthreads();
         int wl = 32;   // width of the last block
         while (wl > 2 && wl / 2 >= n - 32 * (nb - 1)) wl /= 2;
         bool coincident = false;
         const int noff = nb * (nb - 1) / 2;
         // the off-diagonal tiles column by column from the first (full) ones, then the diagonal
-        for (int u = wid; u < noff + nb; u += NW) {
-            int p, q;
-            if (u < noff) {
-                q = 1;
-                while (q * (q + 1) / 2 <= u) ++q;
-                p = u - q * (q - 1) / 2;
-            } else {
-                p = q = u - noff;
-            }
-            const bool diag = p == q;
-            const int w = q == nb - 1 ? wl : 32, in = lane & (w - 1);
-            const int i = 32 * q + in;                                 // this lane's target
-            const int nxt = (lane & ~(w - 1)) | ((lane + 1) & (w - 1));
-            const double *src = S + 32 * p + (diag ? 0 : lane & ~(w - 1));
-            double T[6], A[3] = {0.0, 0.0, 0.0}, J[3] = {0.0, 0.0, 0.0};
-            for (int d = 0; d < 6; ++d) T[d] = S[d * kMaxCluster + i];
-            const int m0 = diag ? 1 : 0, m1 = diag ? w / 2 : w - 1;
+        for (int u0 = 0; u0 < noff + nb; u0 += NW) {
+            const int u = u0 + wid;
+            const bool has = u < noff + nb;   // (uniform over the warp)
+            int p = 0, q = 0, sj = 0, i = 0, w = 32;
+            bool diag = false;
+            double A[3] = {0.0, 0.0, 0.0}, J[3] = {0.0, 0.0, 0.0};
+            if (has) {
+                if (u < noff) {
+                    q = 1;
+                    while (q * (q + 1) / 2 <= u) ++q;
+                    p = u - q * (q - 1) / 2;
+                } else {
+                    p = q = u - noff;
+                }
+                diag = p == q;
+                w = q == nb - 1 ? wl : 32;
+                const int in = lane & (w - 1);
+                i = 32 * q + in;                                           // this lane's target
+                const int nxt = (lane & ~(w - 1)) | ((lane + 1) & (w - 1));
+                const double *src = S + 32 * p + (diag ? 0 : lane & ~(w - 1));
+                double T[6];
+                for (int d = 0; d < 6; ++d) T[d] = S[d * kMaxCluster + i];
+                const int m0 = diag ? 1 : 0, m1 = diag ? w / 2 : w - 1;
 #pragma unroll 1
-            for (int m = m0; m <= m1; ++m) {
-                const bool on = !diag || (lane < w && (m < w / 2 || in < w / 2));
-                pair64_sym<TENSOR>(T, src + ((in + m) & (w - 1)), on, a.pc, A, J, coincident);
-                if (m < m1 || !diag)
+                for (int m = m0; m <= m1; ++m) {
+                    const bool on = !diag || (lane < w && (m < w / 2 || in < w / 2));
+                    pair64_sym<TENSOR>(T, src + ((in + m) & (w - 1)), on, a.pc, A, J, coincident);
+                    if (m < m1 || !diag)
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) J[d] = __shfl_sync(0xffffffffu, J[d], nxt);
+                        for (int d = 0; d < 3; ++d) J[d] = __shfl_sync(0xffffffffu, J[d], nxt);
+                }
+                // off-diagonal: lane l holds source l of block p again; diagonal: source l + w / 2
+                sj = diag ? 32 * p + ((in + m1) & (w - 1)) : 32 * p + lane;
+                if (!diag)
+                    for (int k = w; k < 32; k <<= 1)
+                        for (int d = 0; d < 3; ++d) A[d] += __shfl_xor_sync(0xffffffffu, A[d], k);
             }
-            // off-diagonal: lane l holds source l of block p again; diagonal: source l + w / 2
-            const int sj = diag ? 32 * p + ((in + m1) & (w - 1)) : 32 * p + lane;
-            if (!diag || lane < w)
-                for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + sj] += J[d];
-            __syncwarp();
-            if (!diag)
-                for (int k = w; k < 32; k <<= 1)
-                    for (int d = 0; d < 3; ++d) A[d] += __shfl_xor_sync(0xffffffffu, A[d], k);
-            if (lane < w)
-                for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + i] += A[d];
-            __syncwarp();
+            // a round's tiles add in ascending order, four at a time (each to a sum of its own)
+#pragma unroll
+            for (int turn = 0; turn < NW / kSums64; ++turn) {
+                if (has && wid / kSums64 == turn) {
+                    if (!diag || lane < w)
+                        for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + sj] += J[d];
+                    __syncwarp();
+                    if (lane < w)
+                        for (int d = 0; d < 3; ++d) mine[d * kMaxCluster + i] += A[d];
+                    __syncwarp();
+                }
+                if (NW > kSums64) __syncthreads();
+            }
         }
         if (coincident) atomicOr(a.err, DEV_ERR_COINCIDENT);
         __syncthreads();
         for (int p = tid; p < 3 * n; p += 32 * NW) {
             const int i = p / 3, d = p - 3 * i;
             double V = SUM[d * kMaxCluster + i];
-            for (int k = 1; k < NW; ++k) V += SUM[(3 * k + d) * kMaxCluster + i];
+            for (int k = 1; k < kSums64; ++k) V += SUM[(3 * k + d) * kMaxCluster + i];
             const size_t g = 3 * static_cast<size_t>(o) + p;
             const double nx = a.x64[g] + a.dt * (a.pc.mu0 * __fma_rn(a.pc.c1_d, V, S[(3 + d) * kMaxCluster + i]));
             if (!isfinite(nx)) atomicOr(a.err, DEV_ERR_NONFINITE);
@@ -932,7 +950,7 @@ __global__ void __launch_bounds__(128, 3) batched_sym_kernel(BatchArgs a) {
 // Launch shapes: FP64 -- warps per CTA (one cluster per CTA) x resident CTAs;
 // FP32C -- block of BT = 32 warps threads (R targets each) x resident CTAs.
 static size_t shape_smem(int mode, const BatchShape &sh) {
-    if (mode == MODE_FP64) return batch64_smem(sh.warps);
+    if (mode == MODE_FP64) return batch64_smem();
     if (sh.r == 0) return static_cast<size_t>(sh.warps) * kSymWarpSmem;
     const size_t bt = 32 * static_cast<size_t>(sh.warps);
     const int len = sh.warps == 4 ? (sh.r == 2 ? block_stage_len<128, 2>() : block_stage_len<128, 1>())
