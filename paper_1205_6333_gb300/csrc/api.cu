@@ -129,6 +129,31 @@ static sd_status launch_check(cudaError_t e, const char *what) {
     return SD_OK;
 }
 
+bool vjp_buffers(sd_handle *h, bool create) {
+    if (h->vpartG) return true;
+    const size_t es = h->mode == MODE_FP64 ? sizeof(double) : sizeof(float);
+    // (the product's sums and the VJP's are not live together)
+    size_t g = static_cast<size_t>(h->geomv.maxSlots) * 3 * h->npad * sizeof(double);
+    size_t m = g <= h->part_bytes ? 0 : g;
+    size_t j = h->geomv.sym ? static_cast<size_t>(h->geomv.nT) * 6 * h->geomv.I * es : 0;
+    if (j <= h->jpart_bytes) j = 0;
+    auto up = [](size_t b) { return (b + 255) & ~static_cast<size_t>(255); };
+    h->vwork_bytes = up(g) + up(m) + up(j);
+    if (create && h->vwork_bytes > kVjpEager) return true;
+    // (the call may be recorded into a caller's graph, as it could be when the buffers were
+    // there from the start: an allocation is not part of the capture)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    char *p = static_cast<char *>(dalloc(h, h->vwork_bytes));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (!p) return false;
+    h->vwork = p;
+    h->vpartG = reinterpret_cast<double *>(p);
+    h->vpartM = m ? reinterpret_cast<double *>(p + up(g)) : h->part;
+    h->vjpart = j ? p + up(g) + up(m) : h->jpart;
+    return true;
+}
+
 // ---------------------------------------------------------------- one Euler step
 
 // A Verlet step.  The check kernel writes the mirror, the rebuild request and the clamp
@@ -328,7 +353,7 @@ static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int
         }
         if (e == cudaSuccess) e = launch_vjp_near(h, side, in);
         if (h->verlet && e == cudaSuccess) e = cudaEventRecord(h->ev_join, side);
-        if (e == cudaSuccess) e = launch_vjp_dense(h, st, h->posm, h->frcm, h->wam, h->part, h->part2);
+        if (e == cudaSuccess) e = launch_vjp_dense(h, st, h->posm, h->frcm, h->wam);
         if (h->verlet && e == cudaSuccess) e = cudaStreamWaitEvent(st, h->ev_join, 0);
         if (e == cudaSuccess) e = launch_vjp_epilogue(h, st, in, -1, nullptr, nullptr, dt, h->lam, h->gFacc);
     }
@@ -561,22 +586,18 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out) {
         if (e == cudaSuccess) e = vjp_setup(h);
         if (e == cudaSuccess) e = small_setup(h);
         if (e != cudaSuccess) return fail(SD_ERR_CUDA, std::string("kernel set-up: ") + cudaGetErrorString(e));
-        const int slots = std::max(h->geom.maxSlots, h->geomv.maxSlots);
-        h->part_bytes = static_cast<size_t>(slots) * 3 * h->npad * sizeof(double);
-        h->part2_bytes = static_cast<size_t>(h->geomv.maxSlots) * 3 * h->npad * sizeof(double);
+        h->part_bytes = static_cast<size_t>(h->geom.maxSlots) * 3 * h->npad * sizeof(double);
         h->part = static_cast<double *>(dalloc(h, h->part_bytes));
-        h->part2 = static_cast<double *>(dalloc(h, h->part2_bytes));
         if (h->small.on && (!dalloc_t(h, h->small_sync, 3) || !dalloc_t(h, h->small_xch, 2 * n3)))
             return fail(SD_ERR_OOM, "device allocation of the small systems' exchange");
-        if (!h->part || !h->part2) return fail(SD_ERR_OOM, "device allocation of partial sums");
-        {   // one buffer: the product's and the VJP's source-side sums are not live together
+        if (!h->part) return fail(SD_ERR_OOM, "device allocation of partial sums");
+        if (h->geom.sym) {
             const size_t es = h->mode == MODE_FP64 ? sizeof(double) : sizeof(float);
-            const size_t nd = h->geom.sym ? static_cast<size_t>(h->geom.nT) * 3 * h->geom.I : 0;
-            const size_t nv = h->geomv.sym ? static_cast<size_t>(h->geomv.nT) * 6 * h->geomv.I : 0;
-            h->jpart_bytes = std::max(nd, nv) * es;
-            if (h->jpart_bytes) h->jpart = dalloc(h, h->jpart_bytes);
-            if (h->jpart_bytes && !h->jpart) return fail(SD_ERR_OOM, "device allocation of source-side partial sums");
+            h->jpart_bytes = static_cast<size_t>(h->geom.nT) * 3 * h->geom.I * es;
+            h->jpart = dalloc(h, h->jpart_bytes);
+            if (!h->jpart) return fail(SD_ERR_OOM, "device allocation of source-side partial sums");
         }
+        if (!vjp_buffers(h, true)) return fail(SD_ERR_OOM, "device allocation of partial sums");
     }
 
     // zero everything that padding or defaults rely on
@@ -619,7 +640,7 @@ void sd_destroy(sd_handle *h) {
         dfree(h, m->aos);
         dfree(h, m->soa);
     }
-    void *bufs[] = {h->fext64, h->F64, h->Fa64, h->Wa64, h->part, h->part2, h->jpart,
+    void *bufs[] = {h->fext64, h->F64, h->Fa64, h->Wa64, h->part, h->vwork, h->jpart,
                     h->cl.cell, h->cl.key, h->cl.cnt, h->cl.start, h->cl.bsum, h->cl.sorted,
                     h->ckpt, h->seg, h->lam, h->gFacc, h->near64, h->d_flag, h->d_err,
                     h->near_ent, h->near_out, h->near_n, h->near_off, h->near_cnt, h->vlag, h->xref, h->d_vl,
@@ -1052,6 +1073,7 @@ sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, 
     if (!h->pos_set) return set_error(SD_ERR_STATE, "positions were never set");
     if (h->n == 0) return SD_OK;
     cudaSetDevice(h->device);
+    if (!vjp_buffers(h, false)) return set_error(SD_ERR_OOM, "device allocation of the gradient's partial sums");
     const size_t es = dtype == SD_DTYPE_F32 ? sizeof(float) : sizeof(double);
     const size_t bytes = 3 * es * h->n;
     const void *Fd = F, *Wd = W;
@@ -1075,7 +1097,7 @@ sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, 
     const VjpInput vin{h->x64[h->cur], h->Fa64, h->frcam, h->Wa64, false};
     if (s == SD_OK) s = launch_check(launch_vjp_near(h, h->stream, vin), "near pass");
     if (s == SD_OK)
-        s = launch_check(launch_vjp_dense(h, h->stream, h->posm, h->frcam, h->wam, h->part, h->part2), "vjp kernel");
+        s = launch_check(launch_vjp_dense(h, h->stream, h->posm, h->frcam, h->wam), "vjp kernel");
     if (s == SD_OK)
         s = launch_check(launch_vjp_epilogue(h, h->stream, vin, dtype, gXd, gFd, 0.0, nullptr, nullptr), "vjp epilogue");
     if (s != SD_OK) return s;
@@ -1123,6 +1145,7 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
         sd_status s0 = ensure_seg(h, seg_need, "device allocation of the recompute segment");
         if (s0 != SD_OK) return s0;
     }
+    if (!vjp_buffers(h, false)) return set_error(SD_ERR_OOM, "device allocation of the gradient's partial sums");
     if (!h->lam) {
         if (!dalloc_t(h, h->lam, n3) || !dalloc_t(h, h->gFacc, n3))
             return set_error(SD_ERR_OOM, "device allocation of adjoint vectors");

@@ -255,7 +255,11 @@ struct sd_handle {
     double *Fa64 = nullptr;  sd::Mirror frcam;
     double *Wa64 = nullptr;  sd::Mirror wam;
     double *part = nullptr;  size_t part_bytes = 0;   // dense partial sums
-    double *part2 = nullptr; size_t part2_bytes = 0;  // second output of the VJP kernel
+    // The VJP's partial sums (vjp_buffers): of mu W and of the gradient, and source-side sums.  The
+    // first and the last are the product's own buffers where those are large enough.
+    void *vwork = nullptr;  size_t vwork_bytes = 0;
+    double *vpartM = nullptr, *vpartG = nullptr;
+    void *vjpart = nullptr;
     void *jpart = nullptr;  size_t jpart_bytes = 0;   // symmetric kernels: source-side sums [tile][3][block],
                                                        // float (FP32 modes) or double (FP64)
     sd::DenseGeom geom{}, geomv{};
@@ -382,8 +386,12 @@ cudaError_t launch_small(sd_handle *h, cudaStream_t st, int out, double *x0, dou
                          int f32, void *vout, double dt, int64_t nsteps, int row0, int row1);
 // vjp.cu
 cudaError_t vjp_setup(sd_handle *h);
-cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm, double *partM,
-                             double *partG);
+cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm);
+// The partial-sum buffers, if they are not there yet (false: no memory): up to kVjpEager bytes at
+// creation, larger ones by the first call that needs them, so that a system that never
+// differentiates does not hold them (N = 65,536: 300 MB in FP32C, 1.2 GB in FP64).
+constexpr size_t kVjpEager = size_t(128) << 20;
+bool vjp_buffers(sd_handle *h, bool create);
 // What a vector-Jacobian product is taken of: positions (mirror: posm), forces, cotangents
 // (mirror: wam), and whose candidate list holds the near pairs (vlist: the Verlet steps').
 struct VjpInput {

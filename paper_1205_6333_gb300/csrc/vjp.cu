@@ -588,7 +588,8 @@ __global__ void __launch_bounds__(B) vjp_sym64_kernel(const dbl4 *__restrict__ p
     flush(cur_ib);
 }
 
-// Above this the directed kernels (the source-side sums of the block pairs are 200 MB here).
+// Above this the directed kernels (the source-side sums of the block pairs are 202 MB here in FP32C,
+// 807 MB in FP64).
 constexpr int kVjpSymN = 65536;
 
 // Dynamic shared memory: FP64, two stages of three dbl4 arrays; FP32C, two stages of
@@ -710,9 +711,9 @@ static VjpConst2 vjp_const2(const PairConst &pc) {
     return c;
 }
 
-cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm, double *partM,
-                             double *partG) {
+cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror frcm, Mirror wm) {
     const DenseGeom &g = h->geomv;
+    double *partM = h->vpartM, *partG = h->vpartG;
     const bool f64 = h->mode == MODE_FP64;
     const size_t sym_smem =
         g.sym ? spread_smem(h->num_sms, g.grid, h->vjp_occ, f64 ? 0 : vjp_sym_smem(g.I, g.I / 2), h->vjp_limit) : 0;
@@ -721,7 +722,7 @@ cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror 
         const dbl4 *p = static_cast<const dbl4 *>(posm.aos), *f = static_cast<const dbl4 *>(frcm.aos),
                    *w = static_cast<const dbl4 *>(wm.aos);
         if (g.sym)
-            pick_vjp_sym64(h, g.I)<<<g.grid, g.I, sym_smem, st>>>(p, f, w, partM, partG, static_cast<double *>(h->jpart), h->npad,
+            pick_vjp_sym64(h, g.I)<<<g.grid, g.I, sym_smem, st>>>(p, f, w, partM, partG, static_cast<double *>(h->vjpart), h->npad,
                                                           g, h->pc);
         else
             pick_vjp64(h)<<<g.grid, kNT, vjp_smem(MODE_FP64, g.J), st>>>(p, f, w, partM, partG, h->npad, g, h->pc,
@@ -730,7 +731,7 @@ cudaError_t launch_vjp_dense(sd_handle *h, cudaStream_t st, Mirror posm, Mirror 
         const VjpConst2 c = vjp_const2(h->pc);
         if (g.sym)
             pick_vjp_sym(h, g.I)<<<g.grid, g.I / 2, sym_smem, st>>>(
-                posm.soa, frcm.soa, wm.soa, partM, partG, static_cast<float *>(h->jpart), h->npad, g, c, h->d_err,
+                posm.soa, frcm.soa, wm.soa, partM, partG, static_cast<float *>(h->vjpart), h->npad, g, c, h->d_err,
                 h->watchdog);
         else
             pick_vjp2(h)<<<g.grid, kNT, vjp_smem(MODE_FP32C, g.J), st>>>(posm.soa, frcm.soa, wm.soa, partM, partG,
@@ -1015,9 +1016,9 @@ __global__ void __launch_bounds__(32 * kVjpEpiWarps) vjp_epilogue_kernel(VjpEpiA
 
 static VjpEpiArgs vjp_epi_args(sd_handle *h, const VjpInput &in) {
     VjpEpiArgs a{};
-    a.partM = h->part;
-    a.partG = h->part2;
-    a.jpart = h->jpart;
+    a.partM = h->vpartM;
+    a.partG = h->vpartG;
+    a.jpart = h->vjpart;
     a.npad = h->npad;
     a.g = h->geomv;
     a.x64 = in.x64;
