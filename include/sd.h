@@ -238,10 +238,14 @@ sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, 
  *   gx0 = lambda_0;  gF = dL/dF_ext = sum_n dt mu(x_n) lambda_{n+1}.
  * The forward pass is re-run with FP64 checkpoints every ckpt_every steps
  * (ckpt_every >= 1) and each segment is recomputed once; while the positions of all
- * steps take at most 256 MB (and the memory is there) they are kept instead, and
- * nothing is recomputed.  The handle's positions are restored to x0 on return.  gxT input, gx0 and gF outputs (n x 3 doubles). */
+ * steps take at most 256 MB (sd_set_adjoint_keep; and the memory is there) they are kept
+ * instead, and nothing is recomputed.  Both ways give the same bits.  The handle's
+ * positions are restored to x0 on return.  gxT input, gx0 and gF outputs (n x 3 doubles). */
 sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every, const double *gxT, double *gx0,
                      double *gF, int on_device);
+/* Most bytes of positions sd_adjoint keeps instead of checkpoints (default 256 MB; 0: none, the
+ * memory is then what ckpt_every asks for).  max_bytes >= 0, else SD_ERR_ARG. */
+sd_status sd_set_adjoint_keep(sd_handle *h, int64_t max_bytes);
 
 /* Many independent clusters in one launch per step.  Cluster c holds particles
  * offsets[c] .. offsets[c+1]-1 (offsets: nclusters+1 int32, host memory,

@@ -448,6 +448,10 @@ class System:
         sd_adjoint(self.h, dt, nsteps, ckpt_every, pg, p0, pF, dev)
         return gx0, gF
 
+    def set_adjoint_keep(self, max_bytes):
+        """Most bytes of positions adjoint() keeps instead of checkpoints (0: none)."""
+        _check(lib().sd_set_adjoint_keep(self.h, int(max_bytes)), "sd_set_adjoint_keep")
+
     def profile(self, on=True):
         _check(lib().sd_profile(self.h, int(on)), "sd_profile")
 

@@ -360,10 +360,6 @@ static cudaError_t adjoint_segment(sd_handle *h, cudaStream_t st, double dt, int
     return e;
 }
 
-// Up to this many bytes sd_adjoint keeps the positions of all steps; beyond, checkpoints.
-// (N = 4,096, 40 steps in segments of 20: 3,892 us with two segments recomputed, 3,345 so.)
-constexpr double kKeepBytes = 256.0 * 1024 * 1024;
-
 // Graphs of both parts for a full segment of K steps (the recompute part only when
 // K > 1), cached per (dt, K).
 static sd_status capture_adjoint(sd_handle *h, double dt, int64_t K) {
@@ -1136,7 +1132,8 @@ sd_status sd_adjoint(sd_handle *h, double dt, int64_t nsteps, int32_t ckpt_every
         h->ckpt_bytes = h->ckpt ? need : 0;
         return h->ckpt != nullptr;
     };
-    const bool keep = nsteps > 0 && static_cast<double>(nsteps) * xb <= kKeepBytes && store(static_cast<size_t>(nsteps) * xb);
+    const bool keep = nsteps > 0 && static_cast<double>(nsteps) * xb <= static_cast<double>(h->adj_keep) &&
+                      store(static_cast<size_t>(nsteps) * xb);
     if (!keep && !store(static_cast<size_t>(nck) * xb))
         return set_error(SD_ERR_OOM, "device allocation of checkpoints");
     const bool small = use_small(h);
@@ -1273,6 +1270,18 @@ sd_status sd_profile_read(sd_handle *h, int kernel, double *ms, int64_t *launche
     SD_CUDA(prof_collect(h->prof));
     if (ms) *ms = h->prof.ms[kernel];
     if (launches) *launches = h->prof.launches[kernel];
+    return SD_OK;
+}
+
+sd_status sd_set_adjoint_keep(sd_handle *h, int64_t max_bytes) {
+    if (!h || max_bytes < 0) return set_error(SD_ERR_ARG, "bad handle or number of bytes");
+    h->adj_keep = max_bytes;
+    if (h->ckpt_bytes > static_cast<uint64_t>(max_bytes)) {   // (the next adjoint allocates what it needs)
+        cudaSetDevice(h->device);
+        dfree(h, h->ckpt);
+        h->ckpt = nullptr;
+        h->ckpt_bytes = 0;
+    }
     return SD_OK;
 }
 
