@@ -182,11 +182,14 @@ struct Mirror {
 // bytes: where the grid does not fill them, as much as keeps an SM from taking more than an
 // even share.  (CTAs go where there is room, and beside a kernel on another stream that is
 // here and there at first: an FP64 step of 1,500 particles, 78 CTAs, took 1.25 ms instead of 0.21.)
+// `limit` is allow_smem's: what it leaves of 227 KB is static.
+constexpr size_t kSmemMax = 227 * 1024;
 inline size_t spread_smem(int num_sms, int grid, int occ, size_t need, size_t limit) {
     const size_t per = static_cast<size_t>((grid + num_sms - 1) / num_sms);
     if (per >= static_cast<size_t>(occ)) return need;
     const size_t s = ((228 * 1024 / (per + 1) - 1024) / 128 + 1) * 128;   // (an SM's 228 KB; 1 KB a CTA is the system's)
-    return s < need ? need : (s < limit ? s : limit);
+    const size_t dyn = s > kSmemMax - limit ? s - (kSmemMax - limit) : 0;
+    return dyn < need ? need : (dyn < limit ? dyn : limit);
 }
 // The most dynamic shared memory a launch of fn can have, and the attribute that allows it.  The
 // attribute belongs to the function, which every handle of the process shares: all set-ups
@@ -195,7 +198,7 @@ inline cudaError_t allow_smem(const void *fn, size_t &limit) {
     cudaFuncAttributes at{};
     cudaError_t e = cudaFuncGetAttributes(&at, fn);
     if (e != cudaSuccess) return e;
-    limit = 227 * 1024 - ((at.sharedSizeBytes + 127) & ~static_cast<size_t>(127));
+    limit = kSmemMax - ((at.sharedSizeBytes + 127) & ~static_cast<size_t>(127));
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(limit));
 }
 
