@@ -246,10 +246,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_blocks_kernel(const int *__
     __shared__ int s_warp[33];
     const int base = blockIdx.x * kScanBlock + threadIdx.x * kScanPer;
     int v[kScanPer];
-    for (int k = 0; k < kScanPer; ++k) v[k] = (base + k < H) ? in[base + k] : 0;
+    scan_load(in, base, H, v);
     const int total = block_exclusive_scan<kScanThreads>(v, s_warp);
-    for (int k = 0; k < kScanPer; ++k)
-        if (base + k < H) out[base + k] = v[k];
+    scan_store(out, base, H, v);
     if (threadIdx.x == 0) {
         bsum[blockIdx.x] = total;
         if (gridDim.x == 1) out[H] = total;   // one block: the scan is complete
@@ -324,7 +323,13 @@ cudaError_t launch_build_cells(sd_handle *h, cudaStream_t st, const double *x64,
 // shares the GPU with the all-pairs kernel: 1,024 threads found room only after it.  (A
 // cooperative kernel over all SMs costs some 20 us as a graph node; a build that is certain
 // to run takes the kernels above, faster from N = 16,384 on and as fast below.)
+// What bounds it is a chain of L2 latencies, so a thread's particles and buckets are taken four at
+// a time, their loads and atomics in flight together, and scans move 16 bytes an access: N = 4,096
+// / 16,384 / 32,768 24 / 47 / 84 us one at a time, now 16 / 30 / 51 (cold caches).  The separate
+// kernels take 17 / 25 / 26, of which a step that needs none would pay three to five more launches.
+// Eight at a time are no faster and take 80 registers instead of 64.
 constexpr int kClusterCtas = 8, kClusterThreads = 256, kClusterChunk = kClusterThreads * kScanPer;
+constexpr int kClusterBatch = 4;
 
 __device__ __forceinline__ void cells_barrier() {
     __threadfence();
@@ -338,12 +343,20 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     if ((*vl & 1) == 0) return;   // (uniform over the cluster; vl is the check kernel's)
     __shared__ int s_warp[33];
     const int tid = threadIdx.x, gt = blockIdx.x * kClusterThreads + tid, stride = kClusterCtas * kClusterThreads;
-    for (int i = gt; i < n; i += stride) {
-        const double px = x[3 * i], py = x[3 * i + 1], pz = x[3 * i + 2];
-        xref[3 * i] = px;
-        xref[3 * i + 1] = py;
-        xref[3 * i + 2] = pz;
-        bin_particle(c, i, px, py, pz);
+    constexpr int B = kClusterBatch;
+    for (int i0 = gt; i0 < n; i0 += B * stride) {
+        double p[B][3];
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+            if (i0 + k * stride < n)
+                for (int d = 0; d < 3; ++d) p[k][d] = x[3 * static_cast<size_t>(i0 + k * stride) + d];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const int i = i0 + k * stride;
+            if (i >= n) break;
+            for (int d = 0; d < 3; ++d) xref[3 * static_cast<size_t>(i) + d] = p[k][d];
+            bin_particle(c, i, p[k][0], p[k][1], p[k][2]);
+        }
     }
     if (gt == 0) *list_n = 0;
     cells_barrier();
@@ -351,10 +364,9 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     for (int ch = blockIdx.x; ch < nch; ch += kClusterCtas) {   // scan within each chunk
         const int base = ch * kClusterChunk + tid * kScanPer;
         int v[kScanPer];
-        for (int k = 0; k < kScanPer; ++k) v[k] = base + k < c.H ? c.cnt[base + k] : 0;
+        scan_load(c.cnt, base, c.H, v);
         const int total = block_exclusive_scan<kClusterThreads>(v, s_warp);
-        for (int k = 0; k < kScanPer; ++k)
-            if (base + k < c.H) c.start[base + k] = v[k];
+        scan_store(c.start, base, c.H, v);
         if (tid == 0) {
             c.bsum[ch] = total;
             if (ch == nch - 1) c.start[c.H] = n;   // every particle is in one bucket
@@ -363,16 +375,60 @@ __global__ void __cluster_dims__(kClusterCtas, 1, 1) __launch_bounds__(kClusterT
     cells_barrier();
     if (nch > 1) {
         for (int ch = blockIdx.x; ch < nch; ch += kClusterCtas) {   // ... and the chunks before it
-            int sum = 0;
+            const int base = ch * kClusterChunk + tid * kScanPer;
+            int sum = 0, v[kScanPer];
+            scan_load(c.start, base, c.H, v);
             for (int k = 0; k < ch; ++k) sum += c.bsum[k];
-            for (int k = tid; k < kClusterChunk && ch * kClusterChunk + k < c.H; k += kClusterThreads)
-                c.start[ch * kClusterChunk + k] += sum;
+            for (int k = 0; k < kScanPer; ++k) v[k] += sum;
+            scan_store(c.start, base, c.H, v);
         }
         cells_barrier();
     }
-    for (int i = gt; i < n; i += stride) scatter_particle(c.key, c.start, c.cnt, c.sorted, i, err);
+    for (int i0 = gt; i0 < n; i0 += B * stride) {   // scatter_particle, B at a time
+        uint32_t key[B];
+        int s0[B], s1[B], at[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) key[k] = i0 + k * stride < n ? c.key[i0 + k * stride] : 0u;
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            s0[k] = c.start[key[k]];
+            s1[k] = c.start[key[k] + 1];
+            at[k] = i0 + k * stride < n ? atomicSub(&c.cnt[key[k]], 1) - 1 : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const int i = i0 + k * stride, pos = s0[k] + at[k];
+            if (i >= n) break;
+            if (pos >= s0[k] && pos < s1[k])
+                c.sorted[pos] = i;
+            else
+                atomicOr(err, DEV_ERR_BOUNDS);
+        }
+    }
     cells_barrier();
-    for (int b = gt; b < c.H; b += stride) sort_bucket(c.start, c.sorted, b);
+    for (int b0 = gt; b0 < c.H; b0 += B * stride) {   // sort_bucket, the pairs (nearly all there is to sort) B at a time
+        int s0[B], m[B], u[B], v[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            const int b = b0 + k * stride;
+            s0[k] = b < c.H ? c.start[b] : 0;
+            m[k] = b < c.H ? c.start[b + 1] - s0[k] : 0;
+        }
+#pragma unroll
+        for (int k = 0; k < B; ++k)
+            if (m[k] == 2) {
+                u[k] = c.sorted[s0[k]];
+                v[k] = c.sorted[s0[k] + 1];
+            }
+#pragma unroll
+        for (int k = 0; k < B; ++k) {
+            if (m[k] == 2 && u[k] > v[k]) {
+                c.sorted[s0[k]] = v[k];
+                c.sorted[s0[k] + 1] = u[k];
+            }
+            if (m[k] > 2) sort_bucket(c.start, c.sorted, b0 + k * stride);
+        }
+    }
 }
 
 cudaError_t launch_rebuild_cells(sd_handle *h, cudaStream_t st, const double *x64) {

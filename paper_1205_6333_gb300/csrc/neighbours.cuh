@@ -84,10 +84,10 @@ __device__ __forceinline__ void put_pos_mirror(V4 *m, float *soa, int npad, int 
                wrap_box(pz - x[2], b.L[2], b.invL[2]));
 }
 
+// (the conversion rounds down and saturates by itself: two FP64-rate operations instead of five,
+// which is what a build on a few SMs waits for; then the range is kept for absurd coordinates)
 __device__ __forceinline__ int cell_coord(double x, double inv_h) {
-    double c = floor(x * inv_h);
-    c = fmin(fmax(c, -1.0e9), 1.0e9);  // keep the integer in range for absurd coordinates
-    return static_cast<int>(c);
+    return min(max(__double2int_rd(x * inv_h), -1000000000), 1000000000);
 }
 
 // Cell coordinate in dimension d: nc[d] cells over [0, L) of the wrapped coordinate
@@ -95,7 +95,7 @@ __device__ __forceinline__ int cell_coord(double x, double inv_h) {
 __device__ __forceinline__ int cell_coord_d(const CellList &c, int d, double x) {
     const int nc = c.nc[d];
     if (nc <= 0) return cell_coord(x, c.inv_h);
-    const int k = static_cast<int>(floor(wrap_box(x, c.box.L[d], c.box.invL[d]) * c.box.invL[d] * nc));
+    const int k = __double2int_rd(wrap_box(x, c.box.L[d], c.box.invL[d]) * c.box.invL[d] * nc);
     return k < 0 ? 0 : (k >= nc ? nc - 1 : k);
 }
 
@@ -110,7 +110,21 @@ __device__ __forceinline__ void bin_particle(const CellList &c, int i, double px
     atomicAdd(&c.cnt[k], 1);
 }
 
-constexpr int kScanPer = 16;   // buckets a thread scans
+constexpr int kScanPer = 16;   // buckets a thread scans (both arrays are aligned to 64 bytes and hold whole
+                               // groups of them, 1,024 or a larger power of two: four 16-byte accesses)
+__device__ __forceinline__ void scan_load(const int *in, int base, int H, int (&v)[kScanPer]) {
+#pragma unroll
+    for (int k = 0; k < kScanPer; k += 4) {
+        const int4 q = base < H ? *reinterpret_cast<const int4 *>(in + base + k) : make_int4(0, 0, 0, 0);
+        v[k] = q.x; v[k + 1] = q.y; v[k + 2] = q.z; v[k + 3] = q.w;
+    }
+}
+__device__ __forceinline__ void scan_store(int *out, int base, int H, const int (&v)[kScanPer]) {
+    if (base >= H) return;
+#pragma unroll
+    for (int k = 0; k < kScanPer; k += 4)
+        *reinterpret_cast<int4 *>(out + base + k) = make_int4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+}
 
 // Exclusive scan of kScanPer values per thread across a block; returns the
 // block total.  Warp shuffles within warps, shared memory across warps.
