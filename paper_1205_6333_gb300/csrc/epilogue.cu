@@ -323,6 +323,21 @@ __global__ void __launch_bounds__(128) near_pair_kernel(NearArgs a) {
     if (close && a.flag) atomicOr(a.flag, 1);
 }
 
+// The particles that a full Verlet list left out, corrected again where the step's forces follow the
+// list (soft repulsion, lubrication): the list's build had the forces of the step before.
+template <int TENSOR, int MODE>
+__global__ void __launch_bounds__(128) near_full_kernel(NearArgs a) {
+    if (*a.ent_n <= static_cast<unsigned long long>(a.cap)) return;   // (uniform over the grid)
+    const long long gt = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const long long q = gt / kWalkLanes;
+    const int i = q < a.n ? a.cl.sorted[q] : 0;
+    near_direct<TENSOR, MODE>(a, i, static_cast<int>(gt % kWalkLanes), q < a.n && a.ncnt[i] < 0);
+}
+
+template <int TENSOR, int MODE>
+static void near_launch_full(int nb, cudaStream_t st, const NearArgs &a) {
+    near_full_kernel<TENSOR, MODE><<<nb, 128, 0, st>>>(a);
+}
 template <int TENSOR, int MODE>
 static void near_launch_collect(int nb, cudaStream_t st, const NearArgs &a) {
     near_collect_kernel<TENSOR, MODE, false><<<nb, 128, 0, st>>>(a, nullptr);
@@ -423,6 +438,11 @@ cudaError_t launch_near_pairs(sd_handle *h, cudaStream_t st, const double *x64, 
     const int np = static_cast<int>(std::min<long long>((8LL * h->n + 127) / 128, 2LL * h->num_sms));
     SD_NEAR_DISPATCH(near_launch_pairs, np);
     ++h->launches;
+    if (verlet_step && !h->forces_const) {
+        const int nb = static_cast<int>((static_cast<long long>(h->n) * kWalkLanes + 127) / 128);
+        SD_NEAR_DISPATCH(near_launch_full, nb);
+        ++h->launches;
+    }
     return cudaGetLastError();
 }
 #undef SD_NEAR_DISPATCH
