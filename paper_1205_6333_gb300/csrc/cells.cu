@@ -531,9 +531,11 @@ __global__ void forces_rep_kernel(const double *__restrict__ x, const double *__
 // are added in ascending partner order (entries beyond the cutoff add zeros wherever they
 // stand in the run).  One thread per particle in CTAs of 128 left most SMs idle at small n
 // (N = 4,913, lubrication: 19 us, with four lanes 13; cold caches); from kForceWideN particles
-// on one lane each fills them, and four cost more in the ordered sum (16,384, repulsion: 16 us
-// against 13).
-constexpr int kForceWideN = 8192;
+// on one lane each fills them, and four cost more in the ordered sum.  A step with one lane / four:
+// repulsion at phi = 0.1, N = 8,193 77.4 / 74.7 us, 10,240 98.4 / 96.3, 13,824 142.6 / 141.7, 17,408
+// 204.9 / 205.2; lubrication on a lattice 83.7 / 81.6, 104.9 / 104.5, 147.6 / 149.2, 210.9 / 217.5.
+// The line stands where lubrication's sides meet; both forms give the same bits.
+constexpr int kForceWideN = 10752;
 template <typename V4, int L>
 __global__ void __launch_bounds__(64) forces_list_kernel(const double *__restrict__ x, const double *__restrict__ fext, double gx,
                                    double gy, double gz, double eps, double rc, double s12,

@@ -519,8 +519,10 @@ __device__ __forceinline__ int first_row_at(const DenseGeom &g, int ib, long lon
 #endif
 // Up to SD_EPI_SMALL_N particles the sums are short and the kernel is a chain of dependent
 // loads: eight warps per 32 particles and one particle per lane (more, shorter chains on more
-// SMs), twice the unrolling, and the loads of the tail issued before the sums (16,384: 19.1 ->
-// 17.9 us, cold caches).
+// SMs), twice the unrolling, and the loads of the tail issued before the sums.  A step's epilogue
+// with four warps / eight, cold caches: 12,288 16.3 / 15.3 us, 16,384 19.0 / 17.0, 18,432 20.0 /
+// 18.2, 20,480 21.0 / 30.6, 32,768 20.1 / 29.6: from 19,456 on, four CTAs an SM of 152, the eight
+// warps' CTAs need a second wave.
 #ifndef SD_EPI_SMALL_N
 #define SD_EPI_SMALL_N 16384
 #endif
