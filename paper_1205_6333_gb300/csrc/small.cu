@@ -256,8 +256,7 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
     constexpr int TD = (TENSOR == T_OSEEN) ? T_OSEEN : T_RP;
     constexpr int I = small_block<MODE, R>();
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int2 s_end;   // x: a wait ran out here; y: the step in which one did somewhere in the cluster
-    __shared__ int s_cnt[2];
+    __shared__ int s_end, s_cnt[2];   // s_end: the step in which a wait ran out somewhere in the cluster
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nt = a.nbl * I;                      // targets of this CTA
     const int WB = a.wb;                           // warps per target block
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
     unsigned tag = 0;
     if (!a.solo && a.out == OUT_EULER && a.nsteps > 1) tag = *reinterpret_cast<volatile unsigned *>(a.sync);
     if (tid == 0) {
-        s_end = make_int2(0, 0x7fffffff);
+        s_end = 0x7fffffff;
         s_cnt[0] = s_cnt[1] = 0;
     }
 
@@ -357,8 +356,14 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
                             org[d] = from[d];
                             u[d] = from[3 * static_cast<size_t>(p) + d];
                         }
-                    } else if (!xch_get(a, xb, p, tag + step - 1, org, u)) {
-                        s_end.x = 1;
+                    } else if (!xch_get(a, xb, p, tag + step - 1, org, u) &&
+                               *reinterpret_cast<volatile int *>(&s_end) >= step) {
+                        // A wait ran out.  The cluster has to leave together, since its CTAs store
+                        // into each other's shared memory (padding rows too, which no wait stands
+                        // for): all are told this step before its barrier and leave at the check in
+                        // the next one.  (Told earlier, its peers may be gone.  What the step
+                        // computes from here is of no use, but in bounds.)
+                        for (int r = 0; r < a.nsplit; ++r) cluster_store(cluster_addr(&s_end, r), step);
                     }
                     for (int d = 0; d < 3; ++d) {
                         u[d] -= org[d];
@@ -370,18 +375,9 @@ __global__ void __launch_bounds__(kSmThreads) small_kernel(SmallArgs a) {
             }
         }
         __syncthreads();
-        // A wait ran out here: the cluster has to leave together, since its peers store into
-        // this CTA's shared memory (padding rows too, which no wait stands for).  So every CTA
-        // is told the step before its barrier, this one only meets them there, and all leave at
-        // this place in the next step (y is then the same for all threads: who finds it set
-        // tells nobody, and one told in this very step goes on).
-        const int2 end = s_end;
-        if (end.y < step) break;
-        const bool lost = end.x != 0;
-        if (lost && tid < a.nsplit)
-            cluster_store(cluster_addr(reinterpret_cast<const char *>(&s_end) + sizeof(int), tid), step);
+        if (s_end < step) break;   // (the same for all threads of the cluster: a peer told now writes this step)
         const int nprev = step == 0 ? 0 : s_cnt[cur ^ 1];   // the last step's notes
-        if (mine && !lost) {
+        if (mine) {
             const SmallNear nr{reinterpret_cast<const float *>(s_src), reinterpret_cast<const float *>(s_tgt), s_pd,
                                a.jlen, nt, j0};
             if constexpr (MODE != MODE_FP64) {   // the last step's near pairs at the new positions
