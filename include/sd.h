@@ -79,12 +79,12 @@ typedef enum { SD_DTYPE_F32 = 0, SD_DTYPE_F64 = 1 } sd_dtype;
  *              DIRECTED's, bit for bit; only the order of the sums differs.  The
  *              particles are cut into nb = npad / B blocks (npad = n rounded up
  *              to a multiple of 1024; FP32 modes: B = 512 from npad = 32768 on,
- *              else 256; FP64: B = 128), and the source-side partial sums take
+ *              else 256, or 128 for small n; FP64: B = 128), and the source-side partial sums take
  *              nb (nb + 1) / 2 * 3 B words (FP32 modes: 4-byte, FP64: 8-byte) of
  *              device memory.
  *   AUTO     : SYMMETRIC once there is at least one block pair per two SMs
- *              (nb (nb + 1) / 2 >= SMs / 2; on a 152-SM GB300: n > 2048 in the FP32
- *              modes, n > 1024 in FP64), else DIRECTED. */
+ *              (FP64), or two per SM of blocks of 128 (FP32 modes, small n): on a 152-SM
+ *              GB300 n > 1408 in FP64, n > 3072 in the FP32 modes; else DIRECTED. */
 typedef enum { SD_DENSE_AUTO = 0, SD_DENSE_DIRECTED = 1, SD_DENSE_SYMMETRIC = 2 } sd_dense_kernel;
 
 typedef struct sd_config {
@@ -149,10 +149,10 @@ sd_status sd_create(const sd_config *cfg, sd_handle **out);
 void sd_destroy(sd_handle *h);
 
 /* Positions r_i (n x 3 doubles), copied into the handle's FP64 state; also
- * refreshes the FP32 mirror the all-pairs kernel reads; with Verlet lists it also
- * builds the steps' near-pair list around the new positions (a small system's steps
- * need none, see sd_step), so a trajectory resumed from positions read back continues
- * bit for bit.  Non-finite values give
+ * refreshes the FP32 mirror the all-pairs kernel reads.  With Verlet lists the first
+ * step after it builds the steps' near-pair list afresh (a small system's steps need
+ * none, see sd_step), so a trajectory resumed from positions read back continues bit
+ * for bit.  Non-finite values give
  * SD_ERR_NONFINITE (host pointers: from this call; device pointers: deferred). */
 sd_status sd_set_positions(sd_handle *h, const double *xyz, int on_device);
 sd_status sd_get_positions(sd_handle *h, double *xyz, int on_device);
@@ -163,14 +163,15 @@ sd_status sd_set_forces(sd_handle *h, const double *f, int on_device);
 
 /* Velocities V = mu(x) F at the current positions for the given forces F
  * (n x 3, dtype sd_dtype for both F and V) -- Sec. 2.2, Eq. rotneMobility;
- * Sec. 3.1, step 3.  Does not change the handle's state. */
+ * Sec. 3.1, step 3.  Does not change the handle's state.  V may overlap F. */
 sd_status sd_mobility_apply(sd_handle *h, const void *F, void *V, int dtype, int on_device);
 
 /* nsteps explicit Euler steps (Sec. 3.1): F = F(x_n), v = mu(x_n) F, x_{n+1} = x_n + dt v.
  * Position state is FP64.  Steps run as a replayed CUDA graph on the handle's stream
  * (asynchronous; errors surface at the next synchronising call), or, for a small system
- * with constant forces and dense_kernel AUTO (FP32C n <= 2048, FP64 n <= 1024), up to 512
- * steps per cooperative kernel launch.  nsteps >= 0. */
+ * with constant forces and dense_kernel AUTO (as long as AUTO is DIRECTED: on a 152-SM GB300
+ * FP32C n <= 3072, FP64 n <= 1408; not FP32, nor FP32C boxes so dense that near pairs are
+ * many), up to 512 steps per cooperative kernel launch.  nsteps >= 0. */
 sd_status sd_step(sd_handle *h, double dt, int64_t nsteps);
 
 /* Row shards of the two calls above, for splitting one system over devices by
@@ -228,7 +229,8 @@ sd_status sd_synchronize(sd_handle *h);
 
 /* Vector-Jacobian products of v(x, F) = mu(x) F at the current positions:
  *   gX = (dv/dx)^T W,   gF = mu(x)^T W = mu(x) W     (derivative of Eq. rotneMobility)
- * F, W inputs; gX, gF outputs (n x 3, dtype). */
+ * F, W inputs; gX, gF outputs (n x 3, dtype).  Partial sums of more than 128 MB (n above some
+ * 20,000) are allocated by the first gradient of a handle (SD_ERR_OOM if that fails). */
 sd_status sd_mobility_vjp(sd_handle *h, const void *F, const void *W, void *gX, void *gF, int dtype,
                           int on_device);
 
@@ -259,7 +261,8 @@ sd_status sd_batch_get_positions(sd_batch *b, double *xyz, int on_device);
 sd_status sd_batch_set_forces(sd_batch *b, const double *f, int on_device);
 /* nsteps Euler steps of every cluster: one persistent kernel launch per step,
  * replayed from a CUDA graph.  The launch shape is picked by the built-in
- * autotuner on first use (or by sd_batch_autotune). */
+ * autotuner on first use (or by sd_batch_autotune).  FP64 gives the same bits with every
+ * shape; the FP32C kernels add in orders of their own. */
 sd_status sd_step_batched(sd_batch *b, double dt, int64_t nsteps);
 /* Time the candidate launch shapes on the current state (state unchanged) and keep
  * the fastest.  *choice (may be NULL) receives the index of the chosen shape. */

@@ -55,8 +55,8 @@ cudaError_t launch_stage_pos(sd_handle *h, cudaStream_t st, const double *x64, M
 //     tests them, so the all-pairs kernel need not wait for the near pass.  It is
 //     raised outright when the list may miss pairs: no list yet (bit 2 of vl[0]:
 //     positions never set), overflowed (its particles corrected in place), or a
-//     displacement of skin / 2 or more.  (The list is the steps' own, built when the
-//     positions are set and by the steps' rebuilds; no other pass touches it.)
+//     displacement of skin / 2 or more.  (The list is the steps' own, built by the
+//     first step after the positions are set and by the steps' rebuilds; no other pass touches it.)
 // A thread takes particles and listed pairs in turn over a grid that reaches every SM: one
 // thread walking a particle's run, in CTAs of 256, took 12 us (N = 4,096) to 17 us (4,913
 // on a lattice); now 8 and 9 us, cold caches.

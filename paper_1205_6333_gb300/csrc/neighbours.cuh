@@ -4,35 +4,15 @@
 
 namespace sd {
 
-// Calls f(j) for every particle j != i whose cell is one of the 27 cells around
-// cell ci, in fixed order (cells by offset, bucket entries by index).
 // A neighbour cell coordinate: wrapped in a periodic dimension (nc > 0).
 __device__ __forceinline__ int cell_wrap(int c, int nc) {
     if (nc <= 0) return c;
     return c < 0 ? c + nc : (c >= nc ? c - nc : c);
 }
 
-template <typename Fn>
-__device__ __forceinline__ void for_each_neighbour(const CellList &c, int i, int4 ci, Fn &&f) {
-    for (int oz = -1; oz <= 1; ++oz)
-        for (int oy = -1; oy <= 1; ++oy)
-            for (int ox = -1; ox <= 1; ++ox) {
-                const int cx = cell_wrap(ci.x + ox, c.nc[0]), cy = cell_wrap(ci.y + oy, c.nc[1]),
-                          cz = cell_wrap(ci.z + oz, c.nc[2]);
-                const uint32_t b = cell_hash(cx, cy, cz, c.H);
-                const int s1 = c.start[b + 1];
-                for (int s = c.start[b]; s < s1; ++s) {
-                    const int j = static_cast<int>(dbg_index(c.sorted[dbg_index(s, c.n, c.err)], c.n, c.err));
-                    if (j == i) continue;
-                    const int4 cj = c.cell[j];
-                    if (cj.x != cx || cj.y != cy || cj.z != cz) continue;  // another cell in the same bucket
-                    f(j);
-                }
-            }
-}
-
-// The same walk split over `step` cooperating threads: this thread visits the
-// neighbour cells first, first + step, ... of the 27 (same per-cell order).
+// Calls f(j) for every particle j != i in one of the 27 cells around cell ci, in fixed order
+// (cells by offset, bucket entries by index), split over `step` cooperating threads: this
+// thread visits the cells first, first + step, ...
 template <typename Fn>
 __device__ __forceinline__ void for_each_neighbour_part(const CellList &c, int i, int4 ci, int first, int step,
                                                         Fn &&f) {

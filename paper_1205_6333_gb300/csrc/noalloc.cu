@@ -24,9 +24,10 @@
 // What bounds it is the FP32 pipe.  Two sources share every instruction (the packed
 // f32x2 operations), a thread owns two targets so that a load serves four pairs, and a
 // group of pairs leaves the packed path only where one of them is closer than 2a, so
-// nothing is clamped.  Every pair is evaluated in both directions: using it once
-// (dense_sym_kernel) needs the source-side sums of every tile, 100 MB at n = 65,536,
-// where the scratch array has 12 MB.  Whole call at n = 3,000 / 20,011 / 65,536 with scalar
+// nothing is clamped.  Every pair is evaluated in both directions: using it once, as
+// dense_sym_kernel does, needs the source-side sums of every tile beside the target sums,
+// 50 MB at n = 65,536 with blocks of 512, where the scratch array has 12 MB.  (Up to about
+// 20,000 particles both would fit, 5 + 6 MB; that form is not built.)  Whole call at n = 3,000 / 20,011 / 65,536 with scalar
 // pair terms, one target per thread and eight splits whatever n is: 55 / 570 / 4,844 us;
 // this way 39 / 367 / 3,300 us (22 FP32 operations per ordered pair: 67% of the pipe).
 #include <cmath>

@@ -46,7 +46,7 @@ constexpr int kSmThreads = 32 * kSmWarps + 32;   // ... and one more takes the n
 constexpr int kSmAhead = 64;               // near pairs evaluated ahead (more: after the loop, by all threads)
 constexpr int kSmNotes = 512;              // noted pairs a CTA holds; more: its targets scan their range again
 constexpr double kSmDense = 8192.0;        // expected near pairs (known in a box) from which the near pass's full warps
-                                           // win: an fcc lattice of 2,048 52 us a step here, 48 there; 864: 29 and 41
+                                           // win: an fcc lattice of 2,048 52 us a step here, 35 there; 864: 29 and 41
 constexpr int kSmSoloFP32 = 128;           // largest n one CTA takes (FP32C)
 constexpr int kSmSoloFP64 = 16;            // ... FP64: two FP64 operations a clock and SM, so more SMs sooner
 constexpr int kSmMaxSteps = 512;           // steps per launch
@@ -683,8 +683,8 @@ static void small_config(const sd_handle *h, cudaLaunchConfig_t &cfg, cudaLaunch
 }
 
 // Which systems take this path: the all-pairs kernel left to the library (a caller that
-// names one gets it) and resolved to the directed one (dense_setup: FP32C n <= 2048, FP64
-// n <= 1024; from there on using every pair once pays for the further kernels), and
+// names one gets it) and resolved to the directed one (dense_setup; on 152 SMs FP32C n <= 3,072,
+// FP64 n <= 1,408: from there on using every pair once pays for the further kernels), and
 // forces that do not change with the positions.
 cudaError_t small_setup(sd_handle *h) {
     SmallGeom &g = h->small;

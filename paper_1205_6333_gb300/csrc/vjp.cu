@@ -498,7 +498,8 @@ __global__ void __launch_bounds__(NT) vjp_sym_kernel(const float *__restrict__ p
 // FP64, bound by the FP64 pipe (two operations a clock and SM): 77 operations an unordered
 // pair.  One target per lane; blocks of 32 or 64 particles while there are few, so that the
 // tiles reach every SM.  The sums are divided by c1.  Whole call at
-// N = 200 / 1,500 / 4,096: 397 / 751 / 2,484 us directed, now 112 / 233 / 1,221.
+// N = 200 / 1,500 / 4,096: 397 / 751 / 2,484 us directed, so 112 / 233 / 1,221; since the even
+// spread counts the static arrays, a call waited for takes 224 us at 1,500 (256) and 371 at 2,000 (399).
 template <int TENSOR, bool PER, int B>
 __global__ void __launch_bounds__(B) vjp_sym64_kernel(const dbl4 *__restrict__ pos, const dbl4 *__restrict__ frc,
                                                       const dbl4 *__restrict__ wv, double *__restrict__ partM,
