@@ -1278,6 +1278,7 @@ sd_status sd_set_adjoint_keep(sd_handle *h, int64_t max_bytes) {
     h->adj_keep = max_bytes;
     if (h->ckpt_bytes > static_cast<uint64_t>(max_bytes)) {   // (the next adjoint allocates what it needs)
         cudaSetDevice(h->device);
+        SD_CUDA(cudaStreamSynchronize(h->stream));   // (an adjoint still running reads it)
         dfree(h, h->ckpt);
         h->ckpt = nullptr;
         h->ckpt_bytes = 0;
